@@ -105,9 +105,10 @@ void ata_fused(cudaStream_t s, const SparseView<T>& A, int ncols, int b, const T
 template <typename T>
 void ata_two_phase(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& At, int b, const T* X, T* Y, T* Z,
                    int lanes_a = 0, int lanes_at = 0);
-template <typename T>
-void csr_to_csc(cudaStream_t s, int m, int n, int64_t nnz, const int* rp, const int* ci, const T* va, int* cp,
-                int* ri, T* cv, int* work_n);
+// work: csc_work_ints(n) ints.
+int64_t csc_work_ints(int64_t n);
+void csr_to_csc(cudaStream_t s, int m, int n, int64_t nnz, const int* rp, const int* ci, const double* va, int* cp,
+                int* ri, double* cv, int* work);
 void to_float(cudaStream_t s, int64_t n, const double* a, float* b);
 void col_norms2(cudaStream_t s, int n, const int* cp, const double* cv, double* d);
 void rowptr_check(cudaStream_t s, int m, int64_t nnz, const int64_t* rp64, int* rp32, int* flags);

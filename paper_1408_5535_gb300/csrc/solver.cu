@@ -260,8 +260,8 @@ static void upload_matrix(phsvds_ctx* ctx, Pool& pool, DevA& d, int64_t m, int64
   d.cp = pool.get<int>(n + 1);
   d.ri = pool.get<int>(nnz);
   d.cv = pool.get<double>(nnz);
-  int* work = pool.get<int>(n);
-  csr_to_csc<double>(s, d.m, d.n, nnz, d.rp, d.ci, d.va, d.cp, d.ri, d.cv, work);
+  int* work = pool.get<int>(csc_work_ints(n));
+  csr_to_csc(s, d.m, d.n, nnz, d.rp, d.ci, d.va, d.cp, d.ri, d.cv, work);
   d.A64 = SparseView<double>{d.m, d.n, nnz, d.rp, d.ci, d.va};
   d.At64 = SparseView<double>{d.n, d.m, nnz, d.cp, d.ri, d.cv};
   d.Z64 = pool.get<double>((size_t)m * bmax);
@@ -2841,10 +2841,9 @@ phsvds_status phsvds_csr_to_csc_f64(phsvds_handle h, int64_t m, int64_t n, int64
   if (!h || m < 0 || n < 1 || nnz < 0 || !row_ptr || !csc_ptr) return PHSVDS_ERR_INVALID;
   try {
     CUCHK(cudaSetDevice(h->device));
-    int* work = nullptr;
-    CUCHK(cudaMallocAsync(&work, sizeof(int) * n, h->stream));
-    csr_to_csc<double>(h->stream, (int)m, (int)n, nnz, row_ptr, col_idx, val, csc_ptr, csc_row, csc_val, work);
-    CUCHK(cudaFreeAsync(work, h->stream));
+    Pool pool(h->stream, h->mempool);
+    csr_to_csc(h->stream, (int)m, (int)n, nnz, row_ptr, col_idx, val, csc_ptr, csc_row, csc_val,
+               pool.get<int>(csc_work_ints(n)));
     CUCHK(cudaGetLastError());
   } catch (const PhError& e) {
     return set_err(h, e.st, e.msg);
