@@ -5,8 +5,8 @@
 //
 // Storage is T (double, or float in the mixed-precision stage 1); every
 // product accumulates per thread in T and across thread blocks in FP64.
-// On GB300 the FP64 variants are bound by the FP64 pipe (~1.2 TFLOP/s), the
-// FP32 variants by HBM bandwidth.
+// On GB300 the FP64 pipe (~1.2 TFLOP/s) binds what runs on it; the larger FP64
+// products go to the FP16 tensor cores by exact splitting (k_split.cu).
 #include <algorithm>
 
 #include "common.cuh"
@@ -278,6 +278,13 @@ __global__ void __launch_bounds__(CG_THREADS) k_cgs_pass(int n, Basis<T> P, T* _
   if (n1 + n2) ordered_commit(part, n1, Gout, n2, Tout, rw);
 }
 
+template <typename T>
+static void count_cgs(int n, int p, int q, const double* Gsub, const double* Gout, const double* Tout) {
+  count_work(pcat<T>(PROF_GRAM),
+             2.0 * n * p * q * ((Gsub ? 1 : 0) + (Gout ? 1 : 0)) + (Tout ? (double)n * q * (q + 1) : 0.0),
+             (double)sizeof(T) * n * ((Gsub || Gout ? p : 0) + q * (Gsub ? 2 : 1)));
+}
+
 template <typename T, int Q>
 static void cgs_launch(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, const double* Gsub,
                        double* Gout, double* Tout) {
@@ -301,9 +308,7 @@ static void cgs_launch(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt,
   const RedWs rw = red_ws((size_t)grid * (n1 + n2));
   k_cgs_pass<T, Q><<<grid, CG_THREADS, smem, s>>>(n, P, Tb, ldt, q, Gsub, Gout, Tout, rows, vec, rw); count_launch();
   reduce_partials(s, rw, grid, n1, Gout, n2, Tout);
-  count_work(pcat<T>(PROF_GRAM),
-             2.0 * n * p * q * ((Gsub ? 1 : 0) + (Gout ? 1 : 0)) + (Tout ? (double)n * q * (q + 1) : 0.0),
-             (double)sizeof(T) * n * ((Gsub || Gout ? p : 0) + q * (Gsub ? 2 : 1)));
+  count_cgs<T>(n, p, q, Gsub, Gout, Tout);
 }
 
 template <typename T>
@@ -313,6 +318,11 @@ void cgs_pass(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, c
   ProfScope ps(s, pcat<T>(PROF_GRAM));
   Basis<T> PP = P;
   if (PP.cols() == 0) { Gsub = nullptr; Gout = nullptr; }
+  if constexpr (sizeof(T) == 8)
+    if (cgs_split(s, n, PP, Tb, ldt, q, Gsub, Gout, Tout)) {
+      count_cgs<T>(n, PP.cols(), q, Gsub, Gout, Tout);
+      return;
+    }
   switch (q) {
     case 1: cgs_launch<T, 1>(s, n, PP, Tb, ldt, q, Gsub, Gout, Tout); break;
     case 2: cgs_launch<T, 2>(s, n, PP, Tb, ldt, q, Gsub, Gout, Tout); break;
@@ -326,12 +336,13 @@ void cgs_pass(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, c
 // ---------------------------------------------------------------------------
 constexpr int TS_ROWS = 128;
 constexpr int TS_CB = 8;       // output columns per pass of k_tall_small
-template <typename T>
-__global__ void __launch_bounds__(TS_ROWS) k_tall_small(int n, const T* P, int ldp, int p,
-                                                        const double* __restrict__ Y, int ldy, int r, T* Out,
-                                                        int ldo, const T* __restrict__ Xs, int ldx,
+// FP64 shapes that the tensor-core form does not take (few rows or basis columns).
+__global__ void __launch_bounds__(TS_ROWS) k_tall_small(int n, const double* P, int ldp, int p,
+                                                        const double* __restrict__ Y, int ldy, int r, double* Out,
+                                                        int ldo, const double* __restrict__ Xs, int ldx,
                                                         const double* __restrict__ theta, double* norms2, bool vec,
                                                         RedWs rw) {
+  using T = double;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wn[64][TS_ROWS / 32];                 // per-warp partial norms (fixed order)
   const int rp = (r + TS_CB - 1) / TS_CB * TS_CB;                 // r padded to whole column blocks
@@ -396,28 +407,213 @@ __global__ void __launch_bounds__(TS_ROWS) k_tall_small(int n, const T* P, int l
   }
 }
 
-template <typename T>
-void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
-                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2) {
-  if (n <= 0 || r <= 0) return;
-  ProfScope ps(s, pcat<T>(PROF_TALL));
+static void tall_general(cudaStream_t s, int n, const double* P, int ldp, int p, const double* Y, int ldy, int r,
+                         double* Out, int ldo, const double* Xs, int ldx, const double* theta, double* norms2) {
   int R = TS_ROWS;
   while (R > 32 && (int64_t)ceil_div(n, R) < 2LL * num_sms()) R >>= 1;
   const int rp = (r + TS_CB - 1) / TS_CB * TS_CB;
-  const size_t smem = sizeof(double) * (size_t)((r + 1) & ~1) + sizeof(T) * ((size_t)p * rp + (size_t)p * R);
+  const size_t smem = sizeof(double) * ((size_t)((r + 1) & ~1) + (size_t)p * rp + (size_t)p * R);
   static std::atomic<uint64_t> attr_done{0};
   once_per_device(attr_done, [&] {
-    cudaFuncSetAttribute(k_tall_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_tall_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   });
   int grid = ceil_div(n, R);
   const int cap = num_sms() * 8;
   if (grid > cap) grid = cap;
   const RedWs rw = norms2 ? red_ws((size_t)grid * r) : RedWs{};
-  k_tall_small<T><<<grid, R, smem, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
-                                        cols16(P, ldp), rw); count_launch();
+  k_tall_small<<<grid, R, smem, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2, cols16(P, ldp), rw);
+  count_launch();
   if (norms2) reduce_partials(s, rw, grid, r, norms2, 0, nullptr);
+}
+
+// The same for FP32 storage (any r) and for one or two FP64 columns: RT rows per
+// thread with all their output columns in registers (CB >= r), the basis read
+// straight from memory, coalesced, and the coefficients broadcast from shared
+// memory.  Each basis value is used by one thread only, so staging it would
+// only add a barrier per chunk.  Several rows share a broadcast; with few rows,
+// one per thread spreads them over more SMs.  The norms are summed per thread
+// and reduced once, at the end.  Bound by HBM in FP32 (by latency towards wide
+// outputs, whose sums leave few warps) and by the FP64 pipe in FP64.  Measured
+// against staging with a butterfly per norm: FP32, 155,649 rows, 35 columns to
+// 8 with norms, 46 us -> 19 us (1.6 TB/s; 10 us without norms); 500,000 rows, 35
+// columns to 21, 60 us -> 42 us; FP64, 500,000 rows, 35 columns to 1, 256 us ->
+// 37 us (a staged result takes the FP64 work of 8 columns).
+constexpr int ST_TH = 128;
+
+// FP32 -> FP64 with integer operations (the conversion unit is on GB300's FP64
+// pipe); denormals, Inf and NaN by the ordinary conversion.
+__device__ __noinline__ double widen_special(float f) { return (double)f; }
+__device__ __forceinline__ double widen(float f) {
+  const unsigned b = __float_as_uint(f), m = b & 0x7fffffffu;
+  if (m == 0u) return 0.0;
+  if (m - 0x00800000u >= 0x7f000000u) return widen_special(f);
+  return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// CTAs per SM that the registers are bounded for
+__host__ __device__ constexpr int st_ctas(int regs32) { return regs32 <= 16 ? 8 : regs32 <= 48 ? 5 : 4; }
+
+template <typename T, int CB, int RT, bool NORM>
+__global__ void __launch_bounds__(ST_TH, st_ctas(CB * RT * (int)sizeof(T) / 4)) k_tall_stream(int n, const T* P, int ldp, int p, const double* __restrict__ Y,
+                                                       int ldy, int r, T* Out, int ldo, const T* __restrict__ Xs,
+                                                       int ldx, const double* __restrict__ theta, double* norms2,
+                                                       RedWs rw) {
+  constexpr int UN = RT * CB <= 16 ? 8 : 4;               // basis columns in flight
+  __shared__ __align__(16) T Ys[64 * CB];                 // [p][CB]
+  __shared__ T ths[CB];
+  __shared__ double wn[ST_TH / 32][CB];
+  __shared__ double part[CB];
+  const int tid = threadIdx.x;
+  for (int k = tid; k < p * CB; k += ST_TH) {
+    const int a = k / CB, c = k - a * CB;
+    Ys[k] = c < r ? (T)Y[a + (size_t)c * ldy] : T(0);
+  }
+  for (int c = tid; c < CB; c += ST_TH) ths[c] = theta && c < r ? (T)(-theta[c]) : T(0);
+  __syncthreads();
+  double nr[NORM ? CB : 1];
+#pragma unroll
+  for (int u = 0; u < (NORM ? CB : 1); ++u) nr[u] = 0.0;
+  for (int64_t i0 = (int64_t)blockIdx.x * (ST_TH * RT) + tid; i0 < n; i0 += (int64_t)gridDim.x * (ST_TH * RT)) {
+    // pointers are bumped by a column at a time: offsets of all the columns at
+    // once would take more registers than the sums do
+    T acc[RT][CB];
+    bool ok[RT];
+#pragma unroll
+    for (int v = 0; v < RT; ++v) {
+      ok[v] = i0 + v * ST_TH < n;
+#pragma unroll
+      for (int u = 0; u < CB; ++u) acc[v][u] = T(0);
+    }
+    auto add = [&](const T (&x)[RT], int a) {
+      T yv[CB];
+      lds_vec<T, CB>(Ys + a * CB, yv);
+#pragma unroll
+      for (int v = 0; v < RT; ++v)
+#pragma unroll
+        for (int u = 0; u < CB; ++u) acc[v][u] = fma(x[v], yv[u], acc[v][u]);
+    };
+    const T* src = P + i0;
+    int a = 0;
+#pragma unroll 1
+    for (; a + UN <= p; a += UN) {
+      T x[UN][RT];
+#pragma unroll
+      for (int u = 0; u < UN; ++u) {
+#pragma unroll
+        for (int v = 0; v < RT; ++v) x[u][v] = ok[v] ? src[v * ST_TH] : T(0);
+        src += ldp;
+      }
+#pragma unroll
+      for (int u = 0; u < UN; ++u) add(x[u], a + u);
+    }
+#pragma unroll 1
+    for (; a < p; ++a) {
+      T x[RT];
+#pragma unroll
+      for (int v = 0; v < RT; ++v) x[v] = ok[v] ? src[v * ST_TH] : T(0);
+      src += ldp;
+      add(x, a);
+    }
+    if (theta) {
+      const T* xs = Xs + i0;
+#pragma unroll
+      for (int u = 0; u < CB; ++u) {
+#pragma unroll
+        for (int v = 0; v < RT; ++v)
+          if (u < r && ok[v]) acc[v][u] = fma(ths[u], xs[v * ST_TH], acc[v][u]);
+        xs += ldx;
+      }
+    }
+    T* dst = Out + i0;
+#pragma unroll
+    for (int u = 0; u < CB; ++u) {
+      if (u >= r) break;
+#pragma unroll
+      for (int v = 0; v < RT; ++v)
+        if (ok[v]) {
+          dst[v * ST_TH] = acc[v][u];
+          if constexpr (NORM) {
+            const double w = widen(acc[v][u]);
+            nr[u] = fma(w, w, nr[u]);
+          }
+        }
+      dst += ldo;
+    }
+  }
+  if constexpr (NORM) {
+    constexpr int NP = CB <= 1 ? 1 : CB <= 2 ? 2 : CB <= 4 ? 4 : CB <= 8 ? 8 : CB <= 16 ? 16 : CB <= 32 ? 32 : 64;
+    double v[NP];
+#pragma unroll
+    for (int u = 0; u < NP; ++u) v[u] = u < CB ? nr[u < CB ? u : 0] : 0.0;
+    const int lane = tid & 31;
+    reduce_scatter<double, NP>(v, lane);
+    if constexpr (NP >= 32) {
+#pragma unroll
+      for (int u = 0; u < NP / 32; ++u)
+        if (lane * (NP / 32) + u < CB) wn[tid >> 5][lane * (NP / 32) + u] = v[u];
+    } else {
+      if (lane % (32 / NP) == 0 && lane / (32 / NP) < CB) wn[tid >> 5][lane / (32 / NP)] = v[0];
+    }
+    __syncthreads();
+    for (int c = tid; c < r; c += ST_TH) {
+      double t = 0.0;
+      for (int w = 0; w < ST_TH / 32; ++w) t += wn[w][c];
+      part[c] = t;
+    }
+    __syncthreads();
+    ordered_commit(part, r, norms2, 0, nullptr, rw);
+  }
+}
+
+template <typename T, int CB, int RT>
+static void tall_stream_rt(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
+                           int ldo, const T* Xs, int ldx, const double* theta, double* norms2) {
+  const int grid = std::min(ceil_div(n, ST_TH * RT), num_sms() * 16);
+  if (!norms2) {
+    k_tall_stream<T, CB, RT, false><<<grid, ST_TH, 0, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, nullptr,
+                                                           RedWs{});
+    count_launch();
+    return;
+  }
+  const RedWs rw = red_ws((size_t)grid * r);
+  k_tall_stream<T, CB, RT, true><<<grid, ST_TH, 0, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2, rw);
+  count_launch();
+  reduce_partials(s, rw, grid, r, norms2, 0, nullptr);
+}
+template <typename T, int CB, int RT>
+static void tall_stream(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
+                        int ldo, const T* Xs, int ldx, const double* theta, double* norms2) {
+  // several rows per thread once they leave every SM two CTAs
+  if (RT > 1 && n >= 2 * num_sms() * ST_TH * RT)
+    tall_stream_rt<T, CB, RT>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2);
+  else
+    tall_stream_rt<T, CB, 1>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2);
+}
+
+template <typename T>
+void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
+                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2) {
+  if (n <= 0 || r <= 0) return;
+  ProfScope ps(s, pcat<T>(PROF_TALL));
   count_work(pcat<T>(PROF_TALL), 2.0 * n * p * r + (theta ? 2.0 * n * r : 0.0) + (norms2 ? 2.0 * n * r : 0.0),
              (double)sizeof(T) * n * (p + r + (theta ? r : 0)));
+#define PH_STREAM(CB, RT) return tall_stream<T, CB, RT>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2)
+  if (r == 1) PH_STREAM(1, 1);
+  if constexpr (sizeof(T) == 4) {
+    if (r == 2) PH_STREAM(2, 2);
+    if (r <= 4) PH_STREAM(4, 4);
+    if (r <= 8) PH_STREAM(8, 4);
+    if (r <= 16) PH_STREAM(16, 2);
+    if (r <= 24) PH_STREAM(24, 2);
+    if (r <= 40) PH_STREAM(40, 2);
+    PH_STREAM(64, 1);
+  } else {
+    if (r == 2) PH_STREAM(2, 1);
+    if (tall_split(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2)) return;
+    tall_general(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2);
+  }
+#undef PH_STREAM
 }
 
 // ---------------------------------------------------------------------------

@@ -141,6 +141,13 @@ template <typename T>
 void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
                       int ldo, const T* Xs, int ldx, const double* theta, double* norms2);
 
+// The FP64 forms on the FP16 tensor cores (k_split.cu); false: not a shape
+// for them (nothing launched).
+bool cgs_split(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ldt, int q, const double* Gsub,
+               double* Gout, double* Tout);
+bool tall_split(cudaStream_t s, int n, const double* P, int ldp, int p, const double* Y, int ldy, int r, double* Out,
+                int ldo, const double* Xs, int ldx, const double* theta, double* norms2);
+
 // T <- T * Linv^T  (q x q upper-triangular inverse factor applied on the right,
 // FP64) and copy T into column-major destination Dst (ld ldd) when non-null.
 template <typename T>
