@@ -114,10 +114,10 @@ typedef struct {
     int record_every;
     /* projected eigensolver of stage 1: 0 = FP64 Jacobi spread over an 8-CTA
      * cluster; 1 = one-CTA FP64 Jacobi with each round's work compacted to
-     * its rotating pairs; 2 (default) = an FP32 Jacobi pass, the exact FP64
-     * frame rebuilt from it, and an FP64 Jacobi clean-up of the pairs touching
-     * the targets, whenever the last targets were >= 1e-5 theta_max (FP32
-     * resolves them; GB300's FP64 latency is ~14x its FP32 latency), else 0 */
+     * its rotating pairs; 2 (default) = an FP32 Jacobi pass and a quadratically
+     * convergent FP64 refinement of all pairs, in one launch, whenever the last
+     * targets were >= 1e-5 theta_max (FP32 resolves them; GB300's FP64 latency is
+     * ~14x its FP32 latency), else 0 */
     int projected_solver;
     /* optional initial guess of stage 1 (the hand-off between runs of
      * Sec. 3.3: e.g. the right singular vectors of an earlier solve): host

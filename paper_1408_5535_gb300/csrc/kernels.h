@@ -221,14 +221,18 @@ void jacobi_eig_cluster_ld(cudaStream_t s, int j, double* H, int ldh, double* S,
 void jacobi_eig_fast_ld(cudaStream_t s, int j, double* H, int ldh, double* S, int lds, double* theta, double tol,
                         int max_sweeps, int* sweeps_out, double tol_rel, int ntarget, int tmode, double tshift,
                         int* rot_out);
-// FP64 clean-up after an FP32 pass: Jacobi rotations of the pairs touching
-// the ntarget targets only, to |a_tx| <= tol * max|a_ij|.
-void jacobi_eig_targets_ld(cudaStream_t s, int j, double* H, int ldh, double* S, int lds, double* theta, double tol,
-                           int max_sweeps, int* sweeps_out, int ntarget, int tmode, double tshift, int* rot_out);
 // FP32 bulk pass: Sf (FP64 out) = the FP32 Jacobi rotation diagonalising H to
 // ~tol * ||H||; H is not modified.
 void jacobi_eig32_ld(cudaStream_t s, int j, const double* H, int ldh, double* Sf, int lds, double* theta, double tol,
                      int max_sweeps, int* sweeps_out, int* rot_out);
+// One launch for the Ritz pairs of a stage-1 iteration (k_eig.cu): S (on entry
+// the previous rotation, or ignored when ident; ld as H) becomes orthonormal
+// with S^T H S diagonal to FP64 in the rows of the ntarget smallest (tmode 0) or
+// largest (1) eigenvalues and to FP32 or better elsewhere; theta = the diagonal, order =
+// its ranking, Scols / thcols = the nt first in that order.  counters: FP32
+// sweeps, rotations, refinement steps, steps that rotated.  1 <= j <= 64.
+void eig_step(cudaStream_t s, int j, const double* H, double* S, int ld, bool ident, int ntarget, int tmode, int nt,
+              double* theta, int* order, double* Scols, double* thcols, int* counters);
 void jacobi_svd_ld(cudaStream_t s, int j, double* G, int ldg, double* S, int lds, double* sig, double tol,
                    int max_sweeps, int* sweeps_out);
 void frame_append(cudaStream_t s, int j0, int nb, double* A, int lda, double* S, int lds, const double* Hn);

@@ -32,7 +32,6 @@ constexpr double TOL_MARGIN = 0.9;        // stopping tests use 0.9 delta: the r
 constexpr double JAC_REL = 1e-8;          // relative threshold of the other pairs (they span the restart space)
 constexpr int W_REFRESH = 16;             // stage-1 restarts between recomputations of W = C V
 constexpr double EIG32_GATE = 1e-5;       // FP32-first projected solve when the targets are >= this x theta_max
-constexpr double JAC_REL32 = 1e-6;        // its FP64 clean-up: relative threshold of the non-target pairs
 constexpr int RI_MAXIT = 24;               // stage 2: inverse-iteration steps for the refined vector (at most)
 constexpr double RI_TAU = 1e-10;          // ... which stop once ||R x|| falls by less than this (relative)
 constexpr double STAG_NEAR = 2.0;         // stage-1 stagnation: residual within 2x of its tolerance ...
@@ -434,15 +433,14 @@ static void frame_from_true(cudaStream_t s, int j, const double* Ht, double* S, 
   symmetrise(s, j, Aw, LD);
 }
 
-// Mixed-precision Rayleigh-Ritz eigensolve on GB300 (one SM's FP64 pipe is
-// ~60x slower than its FP32 pipe): an FP32 cyclic Jacobi pass does the large
-// rotations of the warm frame, S <- S Sf is re-orthonormalised and the exact
-// FP64 frame S^T Ht S rebuilt, and (when fp64_cleanup) an FP64 Jacobi pass,
-// tight only on pairs touching the targets, brings the targeted Ritz pairs to
-// FP64 accuracy.  theta = diagonal of the final frame, S = its rotation.
+// Rayleigh-Ritz eigensolve of stage 2 (one target, the closest to tshift): an FP32
+// cyclic Jacobi pass does the large rotations of the warm frame (one SM's FP64
+// pipe is ~60x slower than its FP32 pipe), S <- S Sf is re-orthonormalised and
+// the exact FP64 frame S^T Ht S rebuilt, and an FP64 Jacobi pass, tight only on
+// pairs touching the target, brings the targeted Ritz pair to FP64 accuracy.
+// theta = diagonal of the final frame, S = its rotation.
 static void eig_mixed(cudaStream_t s, int j, const double* Ht, double* S, double* Aw, double* Sf, double* theta,
-                      double* w1, double* w2, bool s_ident, bool fp64_cleanup, int ntarget, int tmode, double tshift,
-                      int* counters, double rel = JAC_REL, bool targets_only = false) {
+                      double* w1, double* w2, bool s_ident, double tshift, int* counters) {
   frame_from_true(s, j, Ht, S, Aw, w1, w2, s_ident ? -1 : 0);
   jacobi_eig32_ld(s, j, Aw, LD, Sf, LD, theta, 1e-6, 30, counters, counters + 1);
   if (s_ident) {
@@ -453,15 +451,8 @@ static void eig_mixed(cudaStream_t s, int j, const double* Ht, double* S, double
     CUCHK(cudaMemcpy2DAsync(S, LD * sizeof(double), w2, LD * sizeof(double), j * sizeof(double), j,
                             cudaMemcpyDeviceToDevice, s));
   }
-  frame_from_true(s, j, Ht, S, Aw, w1, w2, fp64_cleanup ? 2 : 1);
-  if (fp64_cleanup && targets_only)
-    jacobi_eig_targets_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, ntarget, tmode, tshift,
-                          counters + 3);
-  else if (fp64_cleanup)
-    jacobi_eig_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, rel, ntarget, tmode, tshift,
-                  counters + 3);
-  else
-    jacobi_eig32_ld(s, j, Aw, LD, Sf, LD, theta, 1e-6, 0, nullptr, nullptr);  // theta = diag of the rebuilt frame
+  frame_from_true(s, j, Ht, S, Aw, w1, w2, 2);
+  jacobi_eig_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, JAC_REL, 1, 2, tshift, counters + 3);
 }
 
 // Ht = V^T W recomputed from the tall basis after a transform (j x j, FP64
@@ -792,7 +783,7 @@ struct Stage1 {
   std::chrono::steady_clock::time_point t0;
   // device
   T *V, *W, *Xl, *Tb, *Xrm, *Yrm, *Xr, *Rr, *XU;
-  double *Aw, *S, *Ht, *w1, *w2, *Sf, *theta, *Hn, *G1, *G2, *P1, *P2, *M1, *M2, *innorm, *norms, *Scols, *thcols,
+  double *Aw, *S, *Ht, *w1, *w2, *theta, *Hn, *G1, *G2, *P1, *P2, *M1, *M2, *innorm, *norms, *Scols, *thcols,
       *Yt, *A2, *cand, *excl, *sprev, *dots, *thU;
   int *order, *flags, *jn, *idx;
   // host state
@@ -866,7 +857,6 @@ struct Stage1 {
     Ht = pool.get<double>(LD * LD);
     w1 = pool.get<double>(LD * LD);
     w2 = pool.get<double>(LD * LD);
-    Sf = pool.get<double>(LD * LD);
     theta = pool.get<double>(LD);
     Hn = pool.get<double>(LD * 8);
     G1 = pool.get<double>(LD * 8 + LD);
@@ -1017,9 +1007,9 @@ struct Stage1 {
     while (true) {
       check_time();
       if (nb > 0) expand(nb);
-      // projected eigensolve: an FP32 bulk pass and an FP64 clean-up of the
-      // target pairs when the targets are resolvable in FP32, else FP64
-      // Jacobi throughout (GB300's FP64 latency is ~14x its FP32 latency)
+      // projected eigensolve: an FP32 bulk pass and FP64 refinement in one launch
+      // when the targets are resolvable in FP32, else FP64 Jacobi throughout
+      // (GB300's FP64 latency is ~14x its FP32 latency)
       const bool mixed_eig = !bmode && eig_mode == 2 && (largest || eig32_ok);
       const int ntg = bmode ? 0 : std::min(b, k - nlock) + 1;   // B: every pair to the tight threshold
       const int omode = bmode ? 3 : (largest ? 1 : 0);
@@ -1032,16 +1022,15 @@ struct Stage1 {
       // segment without host syncs, replayed as a cached graph
       auto segment = [&]() {
         if (mixed_eig) {
-          eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, sid, true, ntg, largest ? 1 : 0, 0.0, flags + 16, JAC_REL32,
-                    true);
+          eig_step(s, j, Ht, S, LD, sid, ntg, largest ? 1 : 0, nt, theta, order, Scols, thcols, flags + 16);
         } else {
           frame_from_true(s, j, Ht, S, Aw, w1, w2, sid ? -1 : 1);
           (cluster_eig ? jacobi_eig_cluster_ld : jacobi_eig_fast_ld)(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60,
                                                                      flags + 12, JAC_REL, ntg, largest ? 1 : 0, 0.0,
                                                                      flags + 13);
+          order_theta(s, j, theta, omode, 0.0, order);
+          gather_cols(s, j, S, LD, order, nt, Scols, LD, theta, thcols, flags + 14);
         }
-        order_theta(s, j, theta, omode, 0.0, order);
-        gather_cols(s, j, S, LD, order, nt, Scols, LD, theta, thcols, flags + 14);
         tall_times_small<T>(s, n, V, n, j, Scols, LD, nt, Xr, n, nullptr, 0, nullptr, nullptr);
         zero(s, norms, nt);
         tall_times_small<T>(s, n, W, n, j, Scols, LD, nt, Rr, n, Xr, n, thcols, norms);
@@ -1858,7 +1847,7 @@ struct Stage2 {
         if (++restarts > max_restarts) throw PhError{PHSVDS_ERR_NOT_CONVERGED, "stage 2: restart limit reached"};
         // Ritz pairs of H ordered by closeness to the shift (only the
         // restart needs them)
-        eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, s_ident, true, 1, 2, shift, sw + 2);
+        eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, s_ident, shift, sw + 2);
         s_ident = false;
         order_theta(s, j, theta, 2, shift, order);
         // candidates: s1, Ritz vectors by closeness to the shift, then the previous s1

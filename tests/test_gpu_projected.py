@@ -1,0 +1,48 @@
+"""The one-launch projected eigensolve of stage 1 through whole solves: the basis
+orders at which its work division changes (odd and even, below and above 32
+columns, up to 64), both targets, and multiple eigenvalues, against the dense
+SVD."""
+import numpy as np
+import pytest
+
+from paper_1408_5535_gb300 import native, synth
+from tests.gpu_util import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def h():
+    need_gpu()
+    with native.Handle(0) as hh:
+        yield hh
+
+
+@pytest.mark.parametrize("maxb,mins,b,largest", [(4, 2, 1, True), (11, 6, 1, False), (17, 9, 3, True), (32, 20, 1, False),
+                                                 (33, 19, 5, True), (35, 21, 8, False), (56, 30, 8, True),
+                                                 (56, 31, 7, False)])
+def test_triplets_for_every_order_of_the_projected_problem(h, maxb, mins, b, largest):
+    A = synth.random_sparse(300, 150, 6.0, maxb, values="gaussian", shift=0.05)
+    k = min(4, mins - 1)
+    o = native.default_opts(block_size=b, max_basis=maxb, min_restart=mins)
+    sig, U, V, _, st, _ = native.phsvds_solve(h, A.m, A.n, A.row_ptr, A.col, A.val, k,
+                                              native.LARGEST if largest else native.SMALLEST, 1e-14, opts=o)
+    D = A.to_dense()
+    s = np.linalg.svd(D, compute_uv=False)
+    ref = s[:k] if largest else s[::-1][:k]
+    assert np.all(np.abs(sig - ref) <= 1e-10 * ref)
+    res = np.sqrt(np.linalg.norm(D @ V - U * sig, axis=0) ** 2 + np.linalg.norm(D.T @ U - V * sig, axis=0) ** 2)
+    assert np.all(res <= 1e-14 * s[0])
+    assert np.max(np.abs(V.T @ V - np.eye(k))) <= 1e-12
+
+
+def test_multiple_singular_values(h):
+    """Blocks of equal and of nearly equal singular values among the targets."""
+    sigma = np.concatenate([np.repeat([1.0, 1.1], 3), 1.2 + 1e-9 * np.arange(3), np.linspace(1.5, 3.0, 91)])
+    A = synth.givens_diag(200, 100, sigma=sigma, n_rot=150, seed=4)
+    o = native.default_opts(block_size=4)
+    sig, U, V, _, _, _ = native.phsvds_solve(h, A.m, A.n, A.row_ptr, A.col, A.val, 8, native.SMALLEST, 1e-13, opts=o)
+    assert np.all(np.abs(sig - np.sort(sigma)[:8]) <= 1e-10)
+    D = A.to_dense()
+    assert np.all(np.linalg.norm(D @ V - U * sig, axis=0) <= 3e-13)
+    assert np.max(np.abs(V.T @ V - np.eye(8))) <= 1e-11
