@@ -116,36 +116,6 @@ __device__ inline void lds_vec(const T* __restrict__ src, T (&d)[K]) {
   }
 }
 
-// Butterfly reduce-scatter of the N values each lane holds (N a power of two):
-// at the level with lane offset O, a lane keeps the half of its live values
-// selected by its lane bit O and adds the partner's copy of that half, so a
-// warp sum of N values costs N - 1 adds per lane instead of 5 N.  Afterwards
-// (N >= 32) lane l holds the warp sums of values l * (N / 32) + u in v[u],
-// u < N / 32; (N < 32) v[0] of lane l holds the warp sum of value l / (32 / N).
-template <typename T, int N, int O, int CUR>
-__device__ __forceinline__ void reduce_scatter_step(T (&v)[N], int lane) {
-  if constexpr (O > 0) {
-    if constexpr (CUR > 1) {
-      constexpr int H = CUR / 2;
-      const bool up = (lane & O) != 0;
-#pragma unroll
-      for (int i = 0; i < H; ++i) {
-        const T send = up ? v[i] : v[i + H];
-        const T keep = up ? v[i + H] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-      }
-      reduce_scatter_step<T, N, O / 2, H>(v, lane);
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-      reduce_scatter_step<T, N, O / 2, 1>(v, lane);
-    }
-  }
-}
-template <typename T, int N>
-__device__ __forceinline__ void reduce_scatter(T (&v)[N], int lane) {
-  reduce_scatter_step<T, N, 16, N>(v, lane);
-}
-
 // Block CGS pass.  Phase A: all threads load the chunk of P into shared memory
 // (independent loads, so short vectors do not wait on one load per column),
 // then one thread per row applies T -= P Gsub and stores T.  Phase B: warp w

@@ -294,6 +294,17 @@ void s2_step(cudaStream_t s, int64_t N, int nq, const double* Bv, double* v, con
              double* r1, double* r2, double* w1, double* w2, double* t, double* Bw1, double* Bw2, double* Bt,
              const double* x, const double* Bx, double* tbest, double* acc, double* sc, double eta_tol, int patience,
              int maxit);
+// All steps of the block's solve in one launch of one cluster (k_jdsmall.cu), when
+// a step moves at most JD_SMALL_BYTES (false otherwise: nothing launched; the
+// measurements of both sides are in k_jdsmall.cu).
+// After jd_init, with the same vectors: cv n x q, xrm n x width and z m x width
+// scratch (width q padded to 1, 2, 4 or 8); X null in the scaled form; done
+// (device int): the steps taken.
+constexpr double JD_SMALL_BYTES = 26e6;
+template <typename T>
+bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& At, int q, int nq, bool scaled,
+                    const T* Xq, const T* X, const T* ds, const double* theta, T* v, T* u, T* r1, T* r2, T* w1, T* w2,
+                    T* sol, T* cv, T* xrm, T* z, double* sc, int steps, double tol, int* done);
 constexpr int JD2_FIELD_STEPS = 17 * 8 + 5;   // sc index of the steps taken (stage-2 form)
 constexpr int JD_NSCALAR = 17;
 constexpr int JD_FIELD_ACT = 15;   // sc[JD_FIELD_ACT * 8 + c] != 0 while system c iterates

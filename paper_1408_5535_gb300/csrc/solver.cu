@@ -563,6 +563,13 @@ struct GraphCache {
 // projection is applied to the operator's input as well); t = D^{-1/2} y.
 struct InnerSolver {
   int64_t steps = 0, solves = 0;
+  bool pending = false;   // *hstep more steps are to be added (after a synchronisation)
+  int* hstep = nullptr;
+  int64_t taken() {
+    if (pending) steps += *hstep;
+    pending = false;
+    return steps;
+  }
   // Tb (n x q, FP64): residuals on entry, corrections on return.  Xu: the q
   // Ritz vectors, theta (device, q): their Ritz values, Xl: nl locked vectors;
   // dC (device, n): diag(C) for the scaled form (null: unscaled), entries
@@ -583,6 +590,7 @@ struct InnerJD : InnerSolver {
   COp<T> op;
   T *R, *r1, *r2, *v, *sol, *w1, *w2, *X, *Cv, *Xrm, *Yrm, *Xq, *U, *ds;
   double *acc, *sc, *g1;
+  int* nstep;
   GraphCache graphs;
   InnerJD(phsvds_ctx* c, Pool& pool, int n_, int kmax, COp<T> op_, int maxit_, double tol_, bool use_graphs)
       : s(c->stream), n(n_), maxit(maxit_), tol(tol_), op(op_) {
@@ -604,6 +612,8 @@ struct InnerJD : InnerSolver {
     acc = pool.get<double>(32 + 8 * 64);
     sc = pool.get<double>(JD_NSCALAR * 8);
     g1 = pool.get<double>(8 * 64);
+    nstep = pool.get<int>(1);
+    hstep = Host(c).at<int>(20480);   // bytes [20480, 20484), nobody else's
     graphs.enabled = use_graphs;
   }
   // the caller's vectors into the solve's precision, and the result back
@@ -637,6 +647,7 @@ struct InnerJD : InnerSolver {
   void run(phsvds_ctx* ctx, int q, S* Tb, const S* Xu, const double* theta, const S* Xl, int nl, const double* dC,
            double guard) {
     Host h(ctx);
+    taken();   // (the caller has synchronised since the last solve)
     const size_t nq = (size_t)n * q;
     const bool scaled = dC != nullptr;
     in((int64_t)nq, Tb, R);
@@ -654,7 +665,7 @@ struct InnerJD : InnerSolver {
     zero(s, acc, 32);
     jd_colnorms<T>(s, n, q, R, acc);
     jd_init<T>(s, n, q, R, r1, r2, v, sol, w1, w2, acc, sc);
-    const int w = spmm_width(q);
+    const int w = q > 4 ? 8 : q > 2 ? 4 : q;   // every column, padded to a width of the product
     const size_t nacc = 32 + (size_t)8 * nq_;
     Basis<T> P{Xq, n, nq_, nullptr, 0, 0};
     // u: the operator's input (v, or P D^{-1/2} v in the scaled form)
@@ -677,7 +688,15 @@ struct InnerJD : InnerSolver {
     };
     double* hact = h.at<double>(16384);  // bytes [16384, 16448)
     int it = 0;
-    while (it < maxit) {
+    // short vectors: the whole solve is one launch, its step count is read once
+    // the host has synchronised for another reason
+    const bool small = jd_solve_small<T>(s, *op.A, *op.At, q, nq_, scaled, Xq, scaled ? nullptr : X, ds, theta, v, u,
+                                         r1, r2, w1, w2, sol, Cv, Xrm, op.Z, sc, maxit, tol, nstep);
+    if (small) {
+      CUCHK(cudaMemcpyAsync(hstep, nstep, sizeof(int), cudaMemcpyDeviceToHost, s));
+      pending = true;
+    }
+    while (!small && it < maxit) {
       const int m = std::min(chunk, maxit - it);
       graphs.run(s, (3ull << 40) | ((uint64_t)scaled << 32) | ((uint64_t)m << 16) | ((uint64_t)nq_ << 8) | (uint64_t)q,
                  [&]() {
@@ -2153,7 +2172,7 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
     }
     iters32 = s1f.out.iters;
     mv32 = s1f.out.mv;
-    if (jdf) jd32_steps = jdf->steps, jd32_solves = jdf->solves;
+    if (jdf) jd32_steps = jdf->taken(), jd32_solves = jdf->solves;
     jac32[0] = s1f.out.jac_sweeps;
     jac32[1] = s1f.out.jac_rot;
     jac32[2] = s1f.out.jac_calls;
@@ -2329,7 +2348,7 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
     st->fell_back_at = s1.out.fell_back_at;
     st->recorded = s1.out.recorded;
     st->stage1_stagnation_locks = s1.out.stag_locks + stag32;
-    st->inner_steps = (jd ? jd->steps : 0) + jd32_steps;
+    st->inner_steps = (jd ? jd->taken() : 0) + jd32_steps;
     st->inner_solves = (jd ? jd->solves : 0) + jd32_solves;
     st->inner2_steps = inner2_steps;
     st->inner2_solves = inner2_solves;
