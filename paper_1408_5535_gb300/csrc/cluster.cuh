@@ -1,0 +1,113 @@
+// Device and launch helpers of the kernels that keep a whole small problem in one
+// thread-block cluster (k_jdsmall.cu, k_expand.cu).
+#pragma once
+#include <cuda_runtime.h>
+
+#include <atomic>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace ph {
+
+// A row of Q values that another CTA may have written: from L2.
+template <typename T, int Q>
+__device__ __forceinline__ void ld_row(const T* p, T (&r)[Q]) {
+  if constexpr (sizeof(T) * Q % 16 == 0) {
+#pragma unroll
+    for (int k = 0; k < Q; k += 16 / (int)sizeof(T)) {
+      if constexpr (sizeof(T) == 8) {
+        const double2 t = __ldcg(reinterpret_cast<const double2*>(p + k));
+        r[k] = t.x;
+        r[k + 1] = t.y;
+      } else {
+        const float4 t = __ldcg(reinterpret_cast<const float4*>(p + k));
+        r[k] = t.x;
+        r[k + 1] = t.y;
+        r[k + 2] = t.z;
+        r[k + 3] = t.w;
+      }
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) r[k] = __ldcg(p + k);
+  }
+}
+
+// out(row, :) = sum of val * X(col, :) over the entries of rows [r0, r1), L lanes
+// per row, JT threads; row(i, acc) is called by the first lane of the group.
+template <typename T, int Q, int JT, typename F>
+__device__ __forceinline__ void spmm_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
+                                          const T* __restrict__ val, const T* X, int r0, int r1, int L, F&& row) {
+  const int per = JT / L, gl = threadIdx.x % L, gi = threadIdx.x / L;
+  for (int base = r0; base < r1; base += per) {   // uniform trip count: the shuffles need whole warps
+    const int i = base + gi;
+    T acc[Q];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) acc[k] = T(0);
+    if (i < r1) {
+      const int e1 = ptr[i + 1];
+#pragma unroll 4
+      for (int e = ptr[i] + gl; e < e1; e += L) {
+        const int c = idx[e];
+        const T a = val[e];
+        T x[Q];
+        ld_row<T, Q>(X + (size_t)c * Q, x);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) acc[k] = fma(a, x[k], acc[k]);
+      }
+    }
+    for (int o = L / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < Q; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if (i < r1 && gl == 0) row(i, acc);
+  }
+}
+
+// Lanes per row: as many as keep a row within a few rounds of gathers.
+inline int cluster_lanes(double avg) { return avg <= 8.0 ? 1 : avg <= 32.0 ? 4 : 16; }
+
+template <typename A>
+inline cudaLaunchConfig_t cluster_config(A* at, int nc, int threads, size_t smem, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nc);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = nc;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// CTAs of the kernel's cluster on this device: 16 where it can be placed with smem
+// bytes, else 8.  Sets the kernel's attributes (up to smem_max bytes) at first use.
+template <typename K>
+int cluster_size(K kernel, int threads, size_t smem, size_t smem_max, std::atomic<int> (&known)[64]) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int nc = known[dev & 63].load(std::memory_order_acquire);
+  if (nc) return nc;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  nc = 8;
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = cluster_config(at, 16, threads, smem, nullptr);
+  int fit = 0;
+  if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess && fit > 0) nc = 16;
+  cudaGetLastError();
+  known[dev & 63].store(nc, std::memory_order_release);
+  return nc;
+}
+
+template <typename K, typename G>
+void launch_cluster(K kernel, int nc, int threads, size_t smem, cudaStream_t s, const G& args) {
+  cudaLaunchAttribute at[1];
+  const cudaLaunchConfig_t cfg = cluster_config(at, nc, threads, smem, s);
+  cudaLaunchKernelEx(&cfg, kernel, args);
+  count_launch();
+}
+
+}  // namespace ph

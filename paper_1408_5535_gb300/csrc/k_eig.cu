@@ -58,6 +58,7 @@ constexpr double E_SMALL = 0.02;       // m_ij / gap up to which a pair is refin
 // E^2), and a basis transformed by less orthogonal coefficients drifts over the
 // restarts.
 constexpr float E_DONE = 2e-10f;
+constexpr float E_ANGLE = 1e-8f;       // the largest rotation whose square is below eps
 constexpr float J_TOL = 1e-6f;         // FP32 threshold, relative to max |h_ij|
 constexpr int J_SWEEPS = 30;
 
@@ -338,7 +339,11 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
   cl.sync();
   int xb = 0;                                      // the current X
   // ---- refinement
-  const double noise = 2.220446049250313e-16 * mx; // what rounding leaves in B
+  // What rounding leaves in m.  Between nearly equal eigenvalues it gives angles
+  // m / gap of any size that do not shrink from step to step, and each costs its
+  // square of the orthogonality: such a pair is left as it is.
+  const double noise = 4.0 * 2.220446049250313e-16 * mx;
+  bool last = false;                               // this step only makes X orthonormal
   int step = 0, turned = 0;
   float before = INFINITY;
   while (true) {
@@ -407,13 +412,15 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
       const double lr = sm.lam[r], lc = sm.lam[c];
       const double m = fma(-0.5 * (lr + lc), gr, sm.Bc[i][r]), gap = lc - lr;
       double k = 0.0;
-      if (fabs(m) <= E_SMALL * fabs(gap)) {
+      if (last) {
+      } else if (fabs(m) <= E_SMALL * fabs(gap)) {
         if (m != 0.0) {
           // 1 / gap by one Newton step from FP32 (the quotient only has to be
           // good to a share of itself)
           const double gs = gap * down;
           const double y = (double)__frcp_rn((float)gs);
           k = m * down * (y * fma(-gs, y, 2.0));
+          if (fabs(k) > E_ANGLE && fabs(m) <= noise) k = 0.0;
         }
       } else if ((sm.tgt[r] || sm.tgt[c]) && fabs(m) > noise) {
         flag = true;
@@ -524,8 +531,13 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
       continue;
     }
     xb ^= 1;
-    // done, or on the rounding floor of a pair that is nearly one
-    if (!(e > E_DONE) || (e < 1e-7f && e > 0.1f * before) || step >= E_STEPS) break;
+    // done, or on the rounding floor of a pair that is nearly one; what a last large
+    // rotation has cost X is mended by one more step
+    if (last) break;
+    if (!(e > E_DONE) || (e < 1e-7f && e > 0.1f * before) || step >= E_STEPS) {
+      if (!(e > E_ANGLE)) break;
+      last = true;
+    }
     before = e;
   }
   // ---- results
