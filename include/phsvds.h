@@ -93,7 +93,9 @@ typedef struct {
     int rayleigh_ritz;     /* 1 = Algorithm 1 step 3 before stage 2, default 1 */
     uint64_t seed;         /* SplitMix64 seed of the random vectors the method draws */
     double time_limit_s;   /* 0 = none */
-    int profile;           /* 1 = time kernel classes with CUDA events (stats.t_*_ms), default 0 */
+    int profile;           /* 1 = time kernel classes with CUDA events (stats.t_*_ms), default 0;
+                            * what otherwise runs as one launch over several classes then runs
+                            * as its separate kernels */
     /* PHSVDS_PREC_LEARNED: host pointers, copied at the start of the solve.
      * learned_params: PHSVDS_CNN_NPARAM BF16 values; learned_features: 3 planes
      * of n floats (log diffusion, beta_x, beta_y per grid cell); the grid is

@@ -13,7 +13,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libphsvds.so")
-SOURCES = ["k_sparse.cu", "k_tall.cu", "k_split.cu", "k_small.cu", "k_eig.cu", "solver.cu", "batched.cu", "k_cnn.cu", "k_inner.cu", "k_jdsmall.cu"]
+SOURCES = ["k_sparse.cu", "k_tall.cu", "k_split.cu", "k_small.cu", "k_eig.cu", "solver.cu", "batched.cu", "k_cnn.cu", "k_inner.cu", "k_jdsmall.cu", "k_expand.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]

@@ -233,8 +233,9 @@ struct EigArgs {
   const double* H;
   double *S, *theta;
   int* order;
-  double *Scols, *thcols;
+  double *Scols, *thcols, *norms;
   int* counters;
+  const int* skip;
 };
 
 __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(EigArgs g) {
@@ -244,6 +245,8 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
   const int cr = (int)cl.block_rank();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int j = g.j, jj = j + (j & 1), ld = g.ld;
+  if (cr == 0 && tid < g.nt) g.norms[tid] = 0.0;
+  if (*g.skip) return;                             // the same in every CTA, before any barrier
   EigSmem* peer[EC];
 #pragma unroll
   for (int r = 0; r < EC; ++r) peer[r] = cl.map_shared_rank(&sm, r);
@@ -566,13 +569,14 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
 }  // namespace
 
 void eig_step(cudaStream_t s, int j, const double* H, double* S, int ld, bool ident, int ntarget, int tmode, int nt,
-              double* theta, int* order, double* Scols, double* thcols, int* counters) {
+              double* theta, int* order, double* Scols, double* thcols, double* norms,
+              int* counters, const int* skip) {
   ProfScope ps(s, PROF_JACOBI);
   static std::atomic<uint64_t> done{0};
   once_per_device(done, [&] {
     cudaFuncSetAttribute(k_eig_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(EigSmem));
   });
-  EigArgs g{j, ident ? 1 : 0, ntarget, tmode, nt, ld, H, S, theta, order, Scols, thcols, counters};
+  EigArgs g{j, ident ? 1 : 0, ntarget, tmode, nt, ld, H, S, theta, order, Scols, thcols, norms, counters, skip};
   k_eig_step<<<EC, ET, sizeof(EigSmem), s>>>(g);
   count_launch();
 }

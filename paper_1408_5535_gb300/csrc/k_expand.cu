@@ -12,6 +12,20 @@
 //   warps x 4 columns    G = P^T T: lanes over the rows, butterflies in T, CTAs in FP64
 //   rows x LG lanes      T -= P G: LG lanes share the columns of a row
 // Precision is the general form's: partial sums in T over a few rows, FP64 across CTAs.
+//
+// Time per iteration of stage 1 with the general form and with this one (8.5 entries
+// per row of C's factor, 40 basis vectors at most, blocks of 1, 4, 8):
+//   FP64 n =  1000   202 138   350 253   496 359 us
+//        n =  4000   206 150   347 288   488 418
+//        n =  8000   215 171   355 344   541 566
+//        n = 16000   226 214   370 479
+//        n = 32000   245 296
+//   FP32 n =  1000   196 129   312 205   441 294
+//        n = 16000   216 177   348 271   527 418
+//        n = 32000   217 227   359 334   554 528
+//        n = 64000   234 319   389 444   518 567
+// In FP64 the 16 SMs' arithmetic decides (n p b), in FP32 their reads of the basis
+// (n p).  A 2000 x 1000 solve with the defaults: 174 ms -> 121 ms.
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -270,6 +284,7 @@ bool go(cudaStream_t s, ExArgs g) {
   constexpr size_t SMEM_MAX = 200 * 1024;
   g.cap = ((std::max(g.nlock + g.j, g.j + g.nb) + Q) * Q + 1) & ~1;
   g.nc = cluster_size(k_expand_cluster<T, Q>, XT, SMEM_MAX, SMEM_MAX, known);
+  if (g.n <= 2048) g.nc = 8;                       // as fast as 16 at n = 1000 (143 us per iteration both)
   g.rows = ((g.n + g.nc - 1) / g.nc + 1) & ~1;
   const size_t smem = expand_smem(g.nc, g.cap, Q, g.rows, sizeof(T));
   if (smem > SMEM_MAX) return false;
@@ -284,8 +299,11 @@ bool expand_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& A
                   const T* Xl, T* V, T* W, T* Tb, T* xrm, T* z, double* Ht, double* S, double* sprev, int ldh,
                   int* flags, int* bad) {
   const int n = At.nrows, Q = nb > 4 ? 8 : nb > 2 ? 4 : nb;
-  const double work = (double)n * (nlock + j + 8) * Q * 5.0 + 2.0 * A.nnz * Q;
-  if (work > (sizeof(T) == 8 ? EXPAND_WORK64 : EXPAND_WORK32)) return false;
+  // the line (above): in FP64 the cluster's arithmetic, in FP32 its reads of the
+  // basis, and the product's gathers on 16 SMs against what the launches cost
+  const double np = (double)n * (nlock + j + 8);
+  const double bytes = 2.0 * A.nnz * (Q + 2) * sizeof(T);
+  if ((sizeof(T) == 8 ? np * (Q + 1) / 2e6 : np / 1e6) + bytes / (26e6 + 4e6 * Q) > 1.0) return false;
   ProfScope ps(s, sizeof(T) == 4 ? PROF_F32 + PROF_GRAM : PROF_GRAM);
   ExArgs g{};
   g.n = n;

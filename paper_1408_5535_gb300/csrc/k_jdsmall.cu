@@ -17,14 +17,16 @@
 // One cluster has the bandwidth of 16 SMs, about 0.35 TB/s of L2, and a step has 5
 // or 7 barriers of 2 to 3 us with their ramps.  Time of stage 1 per step, general
 // form and this one (four systems, scaled form, weighted grid gradients):
-//   n = 4096 FP32 (3 MB moved)      78 and 27 us    n = 10,000 FP64 (15 MB)  81 and 55 us
-//   n = 32,400 FP32 (24 MB)         84 and 68 us    n = 50,176 FP32 (38 MB)  83 and 82 us
-//   n = 65,536 FP32 (48 MB)         88 and 94 us    n = 32,400 FP64 (47 MB) 118 and 156 us
-// FP32 meets the general form near 38 MB, FP64 near 25 MB; JD_SMALL_BYTES lies at
-// the lower of the two.  A whole solve (10 smallest values, n = 4096) takes 82 ms,
+//   n = 4096 FP32 (3 MB moved)      71 and 29 us    n = 10,000 FP64 (15 MB) 112 and 83 us
+//   n = 16,384 FP64 (24 MB)        114 and 94 us    n = 32,400 FP32 (24 MB)  84 and 68 us
+//   n = 50,176 FP32 (38 MB)         83 and 82 us    n = 65,536 FP32 (48 MB)  88 and 94 us
+//   n = 32,400 FP64 (47 MB)        118 and 156 us
+// FP32 meets the general form near 38 MB, FP64 near 30 MB; JD_SMALL_BYTES lies
+// below both.  A whole solve (10 smallest values, n = 4096) takes 82 ms,
 // with the general form 167 ms.
 #include <cooperative_groups.h>
 
+#include "cluster.cuh"
 #include "common.cuh"
 #include "kernels.h"
 
@@ -71,63 +73,6 @@ __device__ __forceinline__ double wide(float f) {
   return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
 }
 __device__ __forceinline__ double wide(double f) { return f; }
-
-// T of one 8-byte or 4-byte array that another CTA wrote (L2)
-template <typename T>
-__device__ __forceinline__ T ldg2(const T* p) { return __ldcg(p); }
-
-template <typename T, int Q>
-__device__ __forceinline__ void ld_row(const T* p, T (&r)[Q]) {
-  if constexpr (sizeof(T) * Q % 16 == 0) {
-#pragma unroll
-    for (int k = 0; k < Q; k += 16 / (int)sizeof(T)) {
-      if constexpr (sizeof(T) == 8) {
-        const double2 t = __ldcg(reinterpret_cast<const double2*>(p + k));
-        r[k] = t.x;
-        r[k + 1] = t.y;
-      } else {
-        const float4 t = __ldcg(reinterpret_cast<const float4*>(p + k));
-        r[k] = t.x;
-        r[k + 1] = t.y;
-        r[k + 2] = t.z;
-        r[k + 3] = t.w;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < Q; ++k) r[k] = ldg2(p + k);
-  }
-}
-
-// out(row, :) = sum of val * X(col, :) over the entries of rows [r0, r1), L lanes
-// per row; row(i, acc) is called by the first lane of the group.
-template <typename T, int Q, typename F>
-__device__ __forceinline__ void spmm_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
-                                          const T* __restrict__ val, const T* X, int r0, int r1, int L, F&& row) {
-  const int per = JT / L, gl = threadIdx.x % L, gi = threadIdx.x / L;
-  for (int base = r0; base < r1; base += per) {   // uniform trip count: the shuffles need whole warps
-    const int i = base + gi;
-    T acc[Q];
-#pragma unroll
-    for (int k = 0; k < Q; ++k) acc[k] = T(0);
-    if (i < r1) {
-      const int e1 = ptr[i + 1];
-#pragma unroll 4
-      for (int e = ptr[i] + gl; e < e1; e += L) {
-        const int c = idx[e];
-        const T a = val[e];
-        T x[Q];
-        ld_row<T, Q>(X + (size_t)c * Q, x);
-#pragma unroll
-        for (int k = 0; k < Q; ++k) acc[k] = fma(a, x[k], acc[k]);
-      }
-    }
-    for (int o = L / 2; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < Q; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-    if (i < r1 && gl == 0) row(i, acc);
-  }
-}
 
 template <typename T, int Q>
 __global__ void __launch_bounds__(JT, 1) k_jd_cluster(JdArgs g) {
@@ -242,11 +187,11 @@ __global__ void __launch_bounds__(JT, 1) k_jd_cluster(JdArgs g) {
     }
     cl.sync();
     // ---- 3: z = A u
-    spmm_rows<T, Q>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la,
+    spmm_rows<T, Q, JT>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la,
                     [&](int i, const T (&acc)[Q]) { store_row<T, Q>(z + (size_t)i * Q, acc); });
     cl.sync();
     // ---- 4: y = A^T z on the own rows, and its projections
-    spmm_rows<T, Q>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i1, g.lat, [&](int i, const T (&acc)[Q]) {
+    spmm_rows<T, Q, JT>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i1, g.lat, [&](int i, const T (&acc)[Q]) {
 #pragma unroll
       for (int c = 0; c < Q; ++c)
         if (c < q) cv[(size_t)c * n + i] = acc[c];
@@ -390,56 +335,18 @@ __global__ void __launch_bounds__(JT, 1) k_jd_cluster(JdArgs g) {
   cl.sync();                                       // no CTA leaves while a peer may still reach it
 }
 
-// CTAs of the cluster: 16 where the device can place such a cluster, else 8.
 template <typename T, int Q>
 int cluster_ctas() {
-  static std::atomic<int> per_device[64];
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::atomic<int>& known = per_device[dev & 63];
-  int nc = known.load(std::memory_order_acquire);
-  if (nc) return nc;
-  cudaFuncSetAttribute(k_jd_cluster<T, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(JdSmem<T>));
-  cudaFuncSetAttribute(k_jd_cluster<T, Q>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  nc = 8;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(16);
-  cfg.blockDim = dim3(JT);
-  cfg.dynamicSmemBytes = sizeof(JdSmem<T>);
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 16;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int fit = 0;
-  if (cudaOccupancyMaxActiveClusters(&fit, k_jd_cluster<T, Q>, &cfg) == cudaSuccess && fit > 0) nc = 16;
-  cudaGetLastError();
-  known.store(nc, std::memory_order_release);
-  return nc;
+  static std::atomic<int> known[64];
+  return cluster_size(k_jd_cluster<T, Q>, JT, sizeof(JdSmem<T>), sizeof(JdSmem<T>), known);
 }
 
 template <typename T, int Q>
 void go(cudaStream_t s, JdArgs g) {
-  g.nc = cluster_ctas<T, Q>();
-  if (g.n <= 4 * JT) g.nc = 8;                     // a barrier of 8 costs less than the rows gain from 16
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.nc);
-  cfg.blockDim = dim3(JT);
-  cfg.dynamicSmemBytes = sizeof(JdSmem<T>);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = g.nc;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_jd_cluster<T, Q>, g);
-  count_launch();
+  // (a barrier of 8 costs less than short vectors gain from 16)
+  g.nc = std::min(cluster_ctas<T, Q>(), g.n <= 4 * JT ? 8 : 16);
+  launch_cluster(k_jd_cluster<T, Q>, g.nc, JT, sizeof(JdSmem<T>), s, g);
 }
-
-// lanes per row: as many as keep a row within a few rounds of gathers
-int lanes(double avg) { return avg <= 8.0 ? 1 : avg <= 32.0 ? 4 : 16; }
 
 }  // namespace
 
@@ -460,8 +367,8 @@ bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>&
   g.nq = nq;
   g.scaled = scaled;
   g.steps = steps;
-  g.la = lanes(A.avg_row());
-  g.lat = lanes(At.avg_row());
+  g.la = cluster_lanes(A.avg_row());
+  g.lat = cluster_lanes(At.avg_row());
   g.rp = A.ptr;
   g.ci = A.idx;
   g.va = A.val;

@@ -221,6 +221,10 @@ void jacobi_eig_cluster_ld(cudaStream_t s, int j, double* H, int ldh, double* S,
 void jacobi_eig_fast_ld(cudaStream_t s, int j, double* H, int ldh, double* S, int lds, double* theta, double tol,
                         int max_sweeps, int* sweeps_out, double tol_rel, int ntarget, int tmode, double tshift,
                         int* rot_out);
+// FP64 clean-up after an FP32 pass: Jacobi rotations of the pairs touching
+// the ntarget targets only, to |a_tx| <= tol * max|a_ij|.
+void jacobi_eig_targets_ld(cudaStream_t s, int j, double* H, int ldh, double* S, int lds, double* theta, double tol,
+                           int max_sweeps, int* sweeps_out, int ntarget, int tmode, double tshift, int* rot_out);
 // FP32 bulk pass: Sf (FP64 out) = the FP32 Jacobi rotation diagonalising H to
 // ~tol * ||H||; H is not modified.
 void jacobi_eig32_ld(cudaStream_t s, int j, const double* H, int ldh, double* Sf, int lds, double* theta, double tol,
@@ -231,8 +235,9 @@ void jacobi_eig32_ld(cudaStream_t s, int j, const double* H, int ldh, double* Sf
 // largest (1) eigenvalues and to FP32 or better elsewhere; theta = the diagonal, order =
 // its ranking, Scols / thcols = the nt first in that order.  counters: FP32
 // sweeps, rotations, refinement steps, steps that rotated.  1 <= j <= 64.
+// norms[0 .. nt) is zeroed for the sums that follow; with *skip != 0 that is all.
 void eig_step(cudaStream_t s, int j, const double* H, double* S, int ld, bool ident, int ntarget, int tmode, int nt,
-              double* theta, int* order, double* Scols, double* thcols, int* counters);
+              double* theta, int* order, double* Scols, double* thcols, double* norms, int* counters, const int* skip);
 void jacobi_svd_ld(cudaStream_t s, int j, double* G, int ldg, double* S, int lds, double* sig, double tol,
                    int max_sweeps, int* sweeps_out);
 void frame_append(cudaStream_t s, int j0, int nb, double* A, int lda, double* S, int lds, const double* Hn);
@@ -305,6 +310,16 @@ template <typename T>
 bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& At, int q, int nq, bool scaled,
                     const T* Xq, const T* X, const T* ds, const double* theta, T* v, T* u, T* r1, T* r2, T* w1, T* w2,
                     T* sol, T* cv, T* xrm, T* z, double* sc, int steps, double tol, int* done);
+// A block of stage 1 joins the basis in one launch (k_expand.cu): orthonormalises
+// the nb columns of Tb against [Xl | V(:, :j)], then V(:, j:j+nb), W = C V there,
+// the new rows and columns of Ht and S (unit), zero rows j.. of the nsp columns of
+// sprev.  flags[c], flags[nb]: as chol_factor, *bad = flags[nb]; when set, only Tb
+// was written besides.
+// xrm n x 8 and z m x width scratch.  False (nothing launched): too large.
+template <typename T>
+bool expand_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& At, int nb, int nlock, int j, int nsp,
+                  const T* Xl, T* V, T* W, T* Tb, T* xrm, T* z, double* Ht, double* S, double* sprev, int ldh,
+                  int* flags, int* bad);
 constexpr int JD2_FIELD_STEPS = 17 * 8 + 5;   // sc index of the steps taken (stage-2 form)
 constexpr int JD_NSCALAR = 17;
 constexpr int JD_FIELD_ACT = 15;   // sc[JD_FIELD_ACT * 8 + c] != 0 while system c iterates

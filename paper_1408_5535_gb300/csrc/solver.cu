@@ -433,14 +433,16 @@ static void frame_from_true(cudaStream_t s, int j, const double* Ht, double* S, 
   symmetrise(s, j, Aw, LD);
 }
 
-// Rayleigh-Ritz eigensolve of stage 2 (one target, the closest to tshift): an FP32
+// Rayleigh-Ritz eigensolve of stage 2 (one target, the closest to tshift) and, where
+// the kernel classes are timed apart, of stage 1: an FP32
 // cyclic Jacobi pass does the large rotations of the warm frame (one SM's FP64
 // pipe is ~60x slower than its FP32 pipe), S <- S Sf is re-orthonormalised and
 // the exact FP64 frame S^T Ht S rebuilt, and an FP64 Jacobi pass, tight only on
 // pairs touching the target, brings the targeted Ritz pair to FP64 accuracy.
 // theta = diagonal of the final frame, S = its rotation.
 static void eig_mixed(cudaStream_t s, int j, const double* Ht, double* S, double* Aw, double* Sf, double* theta,
-                      double* w1, double* w2, bool s_ident, double tshift, int* counters) {
+                      double* w1, double* w2, bool s_ident, int ntarget, int tmode, double tshift, int* counters,
+                      bool targets_only = false) {
   frame_from_true(s, j, Ht, S, Aw, w1, w2, s_ident ? -1 : 0);
   jacobi_eig32_ld(s, j, Aw, LD, Sf, LD, theta, 1e-6, 30, counters, counters + 1);
   if (s_ident) {
@@ -452,7 +454,12 @@ static void eig_mixed(cudaStream_t s, int j, const double* Ht, double* S, double
                             cudaMemcpyDeviceToDevice, s));
   }
   frame_from_true(s, j, Ht, S, Aw, w1, w2, 2);
-  jacobi_eig_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, JAC_REL, 1, 2, tshift, counters + 3);
+  if (targets_only)
+    jacobi_eig_targets_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, ntarget, tmode, tshift,
+                          counters + 3);
+  else
+    jacobi_eig_ld(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60, counters + 2, JAC_REL, ntarget, tmode, tshift,
+                  counters + 3);
 }
 
 // Ht = V^T W recomputed from the tall basis after a transform (j x j, FP64
@@ -566,10 +573,15 @@ struct InnerSolver {
   bool pending = false;   // *hstep more steps are to be added (after a synchronisation)
   int* hstep = nullptr;
   int64_t taken() {
-    if (pending) steps += *hstep;
+    if (pending) {
+      steps += *hstep;
+      count_work(cls, step_work[0] * *hstep, step_work[1] * *hstep);
+    }
     pending = false;
     return steps;
   }
+  int cls = 0;                        // kernel class and algorithmic flops, bytes of a pending step
+  double step_work[2] = {0.0, 0.0};
   // Tb (n x q, FP64): residuals on entry, corrections on return.  Xu: the q
   // Ritz vectors, theta (device, q): their Ritz values, Xl: nl locked vectors;
   // dC (device, n): diag(C) for the scaled form (null: unscaled), entries
@@ -591,9 +603,11 @@ struct InnerJD : InnerSolver {
   T *R, *r1, *r2, *v, *sol, *w1, *w2, *X, *Cv, *Xrm, *Yrm, *Xq, *U, *ds;
   double *acc, *sc, *g1;
   int* nstep;
+  bool fuse;              // short vectors: one launch per solve (k_jdsmall.cu)
   GraphCache graphs;
-  InnerJD(phsvds_ctx* c, Pool& pool, int n_, int kmax, COp<T> op_, int maxit_, double tol_, bool use_graphs)
-      : s(c->stream), n(n_), maxit(maxit_), tol(tol_), op(op_) {
+  InnerJD(phsvds_ctx* c, Pool& pool, int n_, int kmax, COp<T> op_, int maxit_, double tol_, bool use_graphs,
+          bool fuse_)
+      : s(c->stream), n(n_), maxit(maxit_), tol(tol_), op(op_), fuse(fuse_) {
     const size_t nn = (size_t)n;
     R = pool.get<T>(nn * 8);
     r1 = pool.get<T>(nn * 8);
@@ -690,11 +704,14 @@ struct InnerJD : InnerSolver {
     int it = 0;
     // short vectors: the whole solve is one launch, its step count is read once
     // the host has synchronised for another reason
-    const bool small = jd_solve_small<T>(s, *op.A, *op.At, q, nq_, scaled, Xq, scaled ? nullptr : X, ds, theta, v, u,
-                                         r1, r2, w1, w2, sol, Cv, Xrm, op.Z, sc, maxit, tol, nstep);
+    const bool small = fuse && jd_solve_small<T>(s, *op.A, *op.At, q, nq_, scaled, Xq, scaled ? nullptr : X, ds, theta,
+                                                 v, u, r1, r2, w1, w2, sol, Cv, Xrm, op.Z, sc, maxit, tol, nstep);
     if (small) {
       CUCHK(cudaMemcpyAsync(hstep, nstep, sizeof(int), cudaMemcpyDeviceToHost, s));
       pending = true;
+      cls = sizeof(T) == 4 ? PROF_F32 + PROF_SMALL : PROF_SMALL;
+      step_work[0] = 4.0 * op.A->nnz * q + (double)n * q * (22.0 + nq_ * (scaled ? 8 : 4));
+      step_work[1] = 2.0 * op.A->nnz * (sizeof(T) + 4.0) + sizeof(T) * (double)n * (24.0 * q + nq_ * (scaled ? 4 : 2));
     }
     while (!small && it < maxit) {
       const int m = std::min(chunk, maxit - it);
@@ -805,6 +822,13 @@ struct Stage1 {
   double *Aw, *S, *Ht, *w1, *w2, *theta, *Hn, *G1, *G2, *P1, *P2, *M1, *M2, *innorm, *norms, *Scols, *thcols,
       *Yt, *A2, *cand, *excl, *sprev, *dots, *thU;
   int *order, *flags, *jn, *idx;
+  // the readback of an iteration, laid out as on the host: theta [0, 512), order
+  // [512, 768), norms [768, 832), flags [912, 1104)
+  unsigned char* outb;
+  static constexpr int F0 = 912, FBAD = 40;   // flags' offset; the flag of a deferred check
+  bool fuse = false;      // short vectors: one launch per block (k_expand.cu)
+  bool profile = false;
+  double* Sf = nullptr;
   // host state
   int j = 0, nlock = 0, nsp = 0, rand_ctr = 0;
   bool s_ident = true;
@@ -860,6 +884,10 @@ struct Stage1 {
     cluster_eig = o.projected_solver != 1;
     eig_mode = o.projected_solver;
     graphs.enabled = !o.profile;  // the per-class timing events are not captured
+    // opts.profile times the kernel classes apart, opts.spmm names a schedule
+    profile = o.profile != 0;
+    fuse = !o.profile && o.spmm == PHSVDS_SPMM_AUTO;
+    if (profile) Sf = pool.get<double>(LD * LD);
     stag_window = std::max(100, 6 * (maxb - mins));
     const size_t nn = (size_t)n;
     V = pool.get<T>(nn * maxb);
@@ -876,7 +904,11 @@ struct Stage1 {
     Ht = pool.get<double>(LD * LD);
     w1 = pool.get<double>(LD * LD);
     w2 = pool.get<double>(LD * LD);
-    theta = pool.get<double>(LD);
+    outb = pool.get<unsigned char>(F0 + 48 * sizeof(int));
+    theta = reinterpret_cast<double*>(outb);
+    order = reinterpret_cast<int*>(outb + 512);
+    norms = reinterpret_cast<double*>(outb + 768);
+    flags = reinterpret_cast<int*>(outb + F0);
     Hn = pool.get<double>(LD * 8);
     G1 = pool.get<double>(LD * 8 + LD);
     G2 = pool.get<double>(LD * 8 + LD);
@@ -885,7 +917,6 @@ struct Stage1 {
     M1 = pool.get<double>(64);
     M2 = pool.get<double>(64);
     innorm = pool.get<double>(8);
-    norms = pool.get<double>(8);
     Scols = pool.get<double>(LD * LD);
     thcols = pool.get<double>(LD);
     Yt = pool.get<double>(LD * LD);
@@ -895,8 +926,6 @@ struct Stage1 {
     sprev = pool.get<double>(LD * 8);
     dots = pool.get<double>(16);
     thU = pool.get<double>(8);
-    order = pool.get<int>(LD);
-    flags = pool.get<int>(48);
     jn = pool.get<int>(4);
     idx = pool.get<int>(2 * LD);
     zero(s, sprev, LD * 8);
@@ -939,9 +968,7 @@ struct Stage1 {
       sync(s);
       int* f = h.at<int>(0);
       if (!f[nb]) break;
-      if (attempt >= 3) throw PhError{PHSVDS_ERR_BREAKDOWN, "stage 1: cannot extend the basis"};
-      for (int c = 0; c < nb; ++c)
-        if (f[c]) fill_random<T>(s, n, Tb + (size_t)c * n, seed, RS_BREAK + (uint64_t)(rand_ctr++));
+      refill(nb, f, attempt);
     }
   }
 
@@ -971,8 +998,43 @@ struct Stage1 {
     }
   }
 
-  // Append nb columns (already in Tb) to the basis and the Jacobi frame.
-  void expand(int nb) {
+  // expand's work in one launch; false where it does not apply.
+  bool expand_fused(int nb) {
+    if constexpr (std::is_same_v<Op, COp<T>>) {
+      if (!fuse || !expand_small<T>(s, *op.A, *op.At, nb, nlock, j, nsp, Xl, V, W, Tb, Xrm, op.Z, Ht, S, sprev, LD,
+                                    flags, flags + FBAD))
+        return false;
+      for (int c = nb; c > 0; c -= spmm_width(c)) ++op.calls;
+      return true;
+    }
+    return false;
+  }
+  // the dependent columns of Tb (flags on the host) replaced by random ones
+  void refill(int nb, const int* f, int attempt) {
+    if (attempt >= 3) throw PhError{PHSVDS_ERR_BREAKDOWN, "stage 1: cannot extend the basis"};
+    for (int c = 0; c < nb; ++c)
+      if (f[c]) fill_random<T>(s, n, Tb + (size_t)c * n, seed, RS_BREAK + (uint64_t)(rand_ctr++));
+  }
+
+  // Append nb columns (already in Tb) to the basis and the Jacobi frame.  With
+  // defer, a fused append may return true: its flag FBAD is still to be read, and
+  // if it is set nothing was appended (undo() then, and once more from the start).
+  bool expand(int nb, bool defer = false, int attempt = 0) {
+    Host h(ctx);
+    for (; expand_fused(nb); ++attempt) {
+      if (!defer) {
+        CUCHK(cudaMemcpyAsync(h.at<int>(0), flags, sizeof(int) * (nb + 1), cudaMemcpyDeviceToHost, s));
+        sync(s);
+        const int* f = h.at<int>(0);
+        if (f[nb]) {
+          refill(nb, f, attempt);
+          continue;
+        }
+      }
+      out.mv += nb;
+      j += nb;
+      return defer;
+    }
     orth_append(nb);
     // W's new columns, the new Gram column of H and the frame append: one
     // segment without host syncs (graph-cached)
@@ -988,6 +1050,14 @@ struct Stage1 {
     graphs.run(s, (2ull << 40) | ((uint64_t)nsp << 24) | ((uint64_t)nb << 8) | (uint64_t)j, tail);
     out.mv += nb;
     j += nb;
+    return false;
+  }
+  // After a deferred expand that found dependent columns (hf: the flags): as if it
+  // had not been called, the columns replaced.
+  void undo(int nb, const int* hf) {
+    out.mv -= nb;
+    j -= nb;
+    refill(nb, hf, 0);
   }
 
   // Append more than 8 columns (initial guesses) in chunks.
@@ -1025,11 +1095,12 @@ struct Stage1 {
     int nb = 0;
     while (true) {
       check_time();
-      if (nb > 0) expand(nb);
       // projected eigensolve: an FP32 bulk pass and FP64 refinement in one launch
       // when the targets are resolvable in FP32, else FP64 Jacobi throughout
       // (GB300's FP64 latency is ~14x its FP32 latency)
       const bool mixed_eig = !bmode && eig_mode == 2 && (largest || eig32_ok);
+      const bool one_eig = mixed_eig && !profile;   // opts.profile: its kernels apart
+      const bool pending = nb > 0 && expand(nb, one_eig);
       const int ntg = bmode ? 0 : std::min(b, k - nlock) + 1;   // B: every pair to the tight threshold
       const int omode = bmode ? 3 : (largest ? 1 : 0);
       const int nt = std::min(std::min(b, k - nlock), j);
@@ -1040,29 +1111,37 @@ struct Stage1 {
       // projected eigensolve, Ritz vectors and residuals, readbacks: one
       // segment without host syncs, replayed as a cached graph
       auto segment = [&]() {
-        if (mixed_eig) {
-          eig_step(s, j, Ht, S, LD, sid, ntg, largest ? 1 : 0, nt, theta, order, Scols, thcols, flags + 16);
+        if (one_eig) {
+          eig_step(s, j, Ht, S, LD, sid, ntg, largest ? 1 : 0, nt, theta, order, Scols, thcols, norms, flags + 16,
+                   flags + FBAD);
         } else {
-          frame_from_true(s, j, Ht, S, Aw, w1, w2, sid ? -1 : 1);
-          (cluster_eig ? jacobi_eig_cluster_ld : jacobi_eig_fast_ld)(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60,
-                                                                     flags + 12, JAC_REL, ntg, largest ? 1 : 0, 0.0,
-                                                                     flags + 13);
+          if (mixed_eig) {
+            eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, sid, ntg, largest ? 1 : 0, 0.0, flags + 16, true);
+          } else {
+            frame_from_true(s, j, Ht, S, Aw, w1, w2, sid ? -1 : 1);
+            (cluster_eig ? jacobi_eig_cluster_ld : jacobi_eig_fast_ld)(s, j, Aw, LD, S, LD, theta, JAC_TOL, 60,
+                                                                       flags + 12, JAC_REL, ntg, largest ? 1 : 0, 0.0,
+                                                                       flags + 13);
+          }
           order_theta(s, j, theta, omode, 0.0, order);
           gather_cols(s, j, S, LD, order, nt, Scols, LD, theta, thcols, flags + 14);
         }
         tall_times_small<T>(s, n, V, n, j, Scols, LD, nt, Xr, n, nullptr, 0, nullptr, nullptr);
-        zero(s, norms, nt);
+        if (!one_eig) zero(s, norms, nt);
         tall_times_small<T>(s, n, W, n, j, Scols, LD, nt, Rr, n, Xr, n, thcols, norms);
-        CUCHK(cudaMemcpyAsync(hth, theta, sizeof(double) * j, cudaMemcpyDeviceToHost, s));
-        CUCHK(cudaMemcpyAsync(hord, order, sizeof(int) * j, cudaMemcpyDeviceToHost, s));
-        CUCHK(cudaMemcpyAsync(hn, norms, sizeof(double) * nt, cudaMemcpyDeviceToHost, s));
-        CUCHK(cudaMemcpyAsync(h.at<int>(960), flags + 12, sizeof(int) * 8, cudaMemcpyDeviceToHost, s));
+        CUCHK(cudaMemcpyAsync(h.at<unsigned char>(0), outb, F0 + 48 * sizeof(int), cudaMemcpyDeviceToHost, s));
       };
       const uint64_t key = (uint64_t)j | ((uint64_t)nt << 8) | ((uint64_t)ntg << 16) | ((uint64_t)mixed_eig << 24) |
                            ((uint64_t)sid << 25) | ((uint64_t)bmode << 26);
       graphs.run(s, key, segment);
-      s_ident = false;
       sync(s);
+      if (pending && h.at<int>(F0)[FBAD]) {
+        undo(nb, h.at<int>(F0));
+        expand(nb, false, 1);
+        graphs.run(s, key, segment);
+        sync(s);
+      }
+      s_ident = false;
       out.iters++;
       if (*h.at<int>(968)) throw PhError{PHSVDS_ERR_NAN, "stage 1: corrupted ordering of the Ritz values"};
       if (mixed_eig) {  // FP32 pass + FP64 clean-up
@@ -1866,7 +1945,7 @@ struct Stage2 {
         if (++restarts > max_restarts) throw PhError{PHSVDS_ERR_NOT_CONVERGED, "stage 2: restart limit reached"};
         // Ritz pairs of H ordered by closeness to the shift (only the
         // restart needs them)
-        eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, s_ident, shift, sw + 2);
+        eig_mixed(s, j, Ht, S, Aw, Sf, theta, w1, w2, s_ident, 1, 2, shift, sw + 2);
         s_ident = false;
         order_theta(s, j, theta, 2, shift, order);
         // candidates: s1, Ritz vectors by closeness to the shift, then the previous s1
@@ -2095,6 +2174,7 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
       op32 = tuned_spmm<float>(ctx, pool, A.A32, A.At32, A.Z32, A.n, spmm_width(b), &cached32, o.deterministic);
   }
   const int sch64 = op64.schedule;
+  const bool fuse = !o.profile && o.spmm == PHSVDS_SPMM_AUTO;
   if (st) {
     std::memset(st, 0, sizeof(*st));
     st->spmm_schedule = sch64;
@@ -2149,7 +2229,8 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
     Stage1<float> s1f(ctx, pool, A.n, k, o, largest, tol_in, EPS32, precond1, diag1, op32);
     std::unique_ptr<InnerSolver> jdf;
     if (o.mixed_inner == 2 && (precond1 == PHSVDS_PREC_NONE || precond1 == PHSVDS_PREC_JACOBI)) {
-      jdf = std::make_unique<InnerJD<float>>(ctx, pool, A.n, k, op32, o.inner_maxit, o.inner_tol, !o.profile);
+      jdf = std::make_unique<InnerJD<float>>(ctx, pool, A.n, k, op32, o.inner_maxit, o.inner_tol, !o.profile,
+                                             fuse);
       s1f.jd = jdf.get();
     }
     s1f.lp = &ld;
@@ -2185,7 +2266,8 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
     s1.out.restarts = s1f.out.restarts;
     s1.out.theta_max = s1f.out.theta_max;  // the ||C|| estimate carries over
     if (o.mixed_inner >= 1 && (s1.precond == PHSVDS_PREC_NONE || s1.precond == PHSVDS_PREC_JACOBI)) {
-      jd = std::make_unique<InnerJD<float>>(ctx, pool, A.n, k, op32, o.inner_maxit, o.inner_tol, !o.profile);
+      jd = std::make_unique<InnerJD<float>>(ctx, pool, A.n, k, op32, o.inner_maxit, o.inner_tol, !o.profile,
+                                             fuse);
       s1.jd = jd.get();
     }
     try {
@@ -2198,7 +2280,8 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
     }
   } else {
     if (o.stage1_inner == 1) {
-      jd = std::make_unique<InnerJD<double>>(ctx, pool, A.n, k, op64, o.inner_maxit, o.inner_tol, !o.profile);
+      jd = std::make_unique<InnerJD<double>>(ctx, pool, A.n, k, op64, o.inner_maxit, o.inner_tol, !o.profile,
+                                             fuse);
       s1.jd = jd.get();
     }
     try {
