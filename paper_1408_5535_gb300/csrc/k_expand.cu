@@ -13,8 +13,8 @@
 //   rows x LG lanes      T -= P G: LG lanes share the columns of a row
 // Precision is the general form's: partial sums in T over a few rows, FP64 across CTAs.
 //
-// Time per iteration of stage 1 with the general form and with this one (8.5 entries
-// per row of C's factor, 40 basis vectors at most, blocks of 1, 4, 8):
+// Time per iteration of stage 1 with the general form and with this one (2n x n, 8 entries
+// per row, 35 basis vectors at most, blocks of 1, 4, 8):
 //   FP64 n =  1000   202 138   350 253   496 359 us
 //        n =  4000   206 150   347 288   488 418
 //        n =  8000   215 171   355 344   541 566
