@@ -546,8 +546,12 @@ phsvds_status phsvds_refined_vector_f64(phsvds_handle h, int j, const double* R,
  *   if Gout: Gout += P^T T        (p x q, column-major, leading dim p);
  *   if Tout: Tout += T^T T        (q x q, column-major).
  * Gsub, Gout, Tout are FP64 (each may be NULL); Gout and Tout accumulate, so
- * the caller zeroes them first.  Products accumulate per thread in the
- * storage precision and across thread blocks in FP64.  All pointers DEVICE.
+ * the caller zeroes them first.  FP32 products accumulate per thread in FP32, and
+ * across thread blocks in FP64.  FP64 products of long vectors (n >= 512 and
+ * enough columns) are formed from integer digits on the tensor cores, and every
+ * output that these would not give as well as FP64 multiply-adds is computed by
+ * such: T - P Gsub is within (p + 4) 2^-52 of |T| + |P| |Gsub|, P^T T and T^T T
+ * within (n / 64 + 64) 2^-52 of |P|^T |T| and |T|^T |T|.  All pointers DEVICE.
  * Asynchronous on the handle's stream.  Errors: PHSVDS_ERR_INVALID (nothing
  * launched) for bad sizes or NULL pointers; PHSVDS_ERR_CUDA for a failed launch.
  */
@@ -566,8 +570,9 @@ phsvds_status phsvds_block_cgs_f32(phsvds_handle h, int64_t n, const float* P1, 
  * P n x p (ld ldp >= n, 1 <= p <= 64), Y p x r FP64 (ld ldy >= p,
  * 1 <= r <= 64), Out n x r (ld ldo >= n); theta (r, FP64) and Xs (n x r, ld
  * ldx) may be NULL together (no subtraction); Out may equal P when r <= p (in
- * place).  norms2 (r, FP64, or NULL): norms2[c] += ||Out(:, c)||^2.  All
- * pointers DEVICE; asynchronous.  Errors as phsvds_block_cgs_f64.
+ * place).  norms2 (r, FP64, or NULL): norms2[c] += ||Out(:, c)||^2.  FP64 products
+ * as above: within (p + 4) 2^-52 of |P| |Y|.  All pointers DEVICE; asynchronous.
+ * Errors as phsvds_block_cgs_f64.
  */
 phsvds_status phsvds_tall_small_f64(phsvds_handle h, int64_t n, const double* P, int ldp, int p, const double* Y,
                                     int ldy, int r, double* Out, int ldo, const double* Xs, int ldx,

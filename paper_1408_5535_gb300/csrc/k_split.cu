@@ -7,14 +7,24 @@
 // 8 bits (Ozaki, Ogita, Oishi, Rump, "Error-free transformations of matrix
 // multiplication", Numer. Algorithms 59, 2012; the digits are integers, as in
 // the INT8 variants of that scheme, but held in FP16).  The products of two
-// digits are exact in FP16 x FP16 -> FP32, and so are their sums: |digit| <=
-// 128, at most 64 terms of at most 4 digit pairs stay within 2^22, and every
-// accumulator starts at 1.5 * 2^23, where FP32 counts in ones, so that its bits
-// are the integer sum.  Digit pairs (s, t) with s + t <= 7 are kept (36 of 64);
-// the sums of all orders are put together as one 64-bit integer and rounded to
-// FP64 once.  The error is at most 2^-54 of (row maximum) x (column maximum) x
-// terms, which is below that of a chain of FP64 multiply-adds (relative to the
-// 64-bit values, p = 35, r = 21: 5e-17 against 2e-16).
+// digits are exact in FP16 x FP16 -> FP32, and so are their sums: over at most
+// 64 terms an accumulator stays within 2^22 (acc_of), and every accumulator
+// starts at 1.5 * 2^23, where FP32 counts in ones, so that its bits are the
+// integer sum.  Digit pairs (s, t) with s + t <= 7 are kept (36 of 64); the sums
+// of all orders are put together as one 64-bit integer and rounded to FP64 once.
+//
+// Accuracy.  What is cut off is relative to (row maximum) x (column maximum): with
+// integers M, N below 2^62, each of K terms loses at most 2 * 2^62 by the cuts of M
+// and N and 7.1 * 2^62 by the dropped pairs, the sum 2^67 by its last place, K * 2^65.2
+// + 2^67 in all.  A chain of FP64 multiply-adds is relative to the sum of the moduli,
+// S = sum |M N|, which may lie far below: P(i,:) = (1e25, 1, 1, ..) times (0, 1, 1, ..).
+// So one more product per step adds up the moduli of the leading digits (FP16
+// accumulators, saturating).  |M| >= 0.498 * 2^56 |leading digit|, so a sum of
+// 2^8 proves S >= 2^118 and the error below (K + 4) 2^-52 S; an output that does not
+// reach it is computed in FP64 from the tile in shared memory (redo).  What is kept is in
+// fact better than the chain: random values with p = 8 to 64: at most 0.5 eps S, mean
+// 0.04, against 2.5 and 0.18; with identity-like coefficients, where a quarter is
+// computed anew, at most 1.0 and mean 0.20 against 6.5 and 0.79.
 //
 // Why mma.sync: a tile's contraction is 16 x 8 x 64 per digit pair and its
 // operands are made in registers by the warp that uses them, so a warp-level
@@ -25,8 +35,10 @@
 // either's rate: the two take turns within a warp, and 16 warps fit an SM.
 //
 // Measured on the FP64 pipe and here: Gram-Schmidt pass, 500,000 x 55 against 8,
-// subtract and project, 801 us -> 220 us (ncu: integer pipe 51%, tensor 30%);
-// V Y, 500,000 x 35 to 21, 694 us -> 173 us (tensor 52%); to 8, 265 us -> 75 us.
+// subtract and project, 796 us -> 225 us; V Y, 500,000 x 35 to 21, 694 us -> 173 us; to
+// 8, 265 us -> 79 us (without the sums of moduli 218, 173 and 74 us).  Where outputs are
+// computed anew it takes longer: V Y with coefficients I + 1e-3 noise 415 us; the pass
+// on log-normal(2) elements 542 us; elements over 10 decades 705 to 850 us.
 //
 // A tile with an Inf, a NaN or values below 2^-950 is computed in plain FP64.
 #include <algorithm>
@@ -95,10 +107,23 @@ __device__ __forceinline__ void digits2(double x0, int base0, double x1, int bas
 }
 
 // The accumulator of the digit pair (s, t): orders s + t = 0..4 have one
-// each, 5, 6 and 7 two each (at most 4 pairs per accumulator).
+// each, 5, 6 and 7 two each.  The leading digit of a 62-bit integer is at most 64 in
+// modulus, the others 128: four pairs of these, or five with two leading digits among
+// them (order 4), over 64 terms are at most 2^22.
 __host__ __device__ constexpr int acc_of(int s, int t) {
   return s + t <= 4 ? s + t : s + t == 5 ? (s < 3 ? 5 : 6) : s + t == 6 ? (s < 4 ? 7 : 8) : (s < 4 ? 9 : 10);
 }
+constexpr bool acc_fits() {
+  for (int k = 0; k < NACC; ++k) {
+    int most = 0;
+    for (int a = 0; a < NS; ++a)
+      for (int b = 0; a + b < NS; ++b)
+        if (acc_of(a, b) == k) most += 64 * (a ? 128 : 64) * (b ? 128 : 64);
+    if (most > 1 << 22) return false;
+  }
+  return true;
+}
+static_assert(acc_fits(), "an accumulator would leave the binade in which FP32 counts in ones");
 
 __device__ __forceinline__ void mma16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -144,6 +169,85 @@ __device__ __forceinline__ double times_pow2(long long k, int D) {
   return scalbn(v, D);
 }
 constexpr int E_OUT = 2101;            // value = sum * 2^(base_a + base_b - E_OUT)
+
+// Sums of the moduli of the leading digits, beside the products (16 x 8, FP16).
+struct Mag {
+  unsigned c[2];
+  __device__ __forceinline__ void clear() { c[0] = c[1] = 0u; }
+  __device__ __forceinline__ void add(unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+    constexpr unsigned ABS = 0x7fff7fffu;
+    asm("mma.sync.aligned.m16n8k16.row.col.f16.f16.f16.f16 {%0,%1}, {%2,%3,%4,%5}, {%6,%7}, {%0,%1};"
+        : "+r"(c[0]), "+r"(c[1])
+        : "r"(a0 & ABS), "r"(a1 & ABS), "r"(a2 & ABS), "r"(a3 & ABS), "r"(b0 & ABS), "r"(b1 & ABS));
+  }
+  // biased exponents of the sums of outputs 2 h and 2 h + 1 (k + 15 for 2^k, 0 for no sum), in halves
+  __device__ __forceinline__ unsigned levels(int h) const { return (c[h] >> 10) & 0x001f001fu; }
+};
+constexpr unsigned MAG_MIN = (8 + 15) * 0x10001u;   // sums of 2^8 and more
+// bits 0, 1: a half of v is below that of w
+__device__ __forceinline__ unsigned less2(unsigned v, unsigned w) {
+  return ((v & 0xffffu) < (w & 0xffffu) ? 1u : 0u) | ((v >> 16) < (w >> 16) ? 2u : 0u);
+}
+// whether either half of any of the warp's v is below that of its w
+__device__ __forceinline__ bool any_less2(unsigned v, unsigned w) {
+  return __any_sync(0xffffffffu, __vmaxu2(v, w) != v);
+}
+
+// out[i] = sum over k < len of x(a, k) y(b, k) in FP64 for the outputs i of the lane's
+// bits in need, a = g + 8 (i / 2), b = 2 t + i % 2 (strides xa, xk, yb, yk).  The warp
+// shares the work: as many lanes per output as there are outputs for.  A multiply-add
+// holds the SM's FP64 pipe for 16 clocks whatever the lanes in use, so a few outputs take
+// a tenth of the tile's FP64 time.  list: 128 bytes of the warp.  Returns how many there are.
+__device__ __noinline__ int redo_list(unsigned need, const double* x, int xa, int xk, const double* y, int yb, int yk,
+                                      int len, unsigned char* list, double* fix) {
+  const int lane = threadIdx.x & 31;
+  int at[4], total = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool mine = (need >> i) & 1u;
+    const unsigned m = __ballot_sync(0xffffffffu, mine);
+    at[i] = total + __popc(m & ((1u << lane) - 1u));
+    if (mine) list[at[i]] = (unsigned char)(i * 32 + lane);
+    total += __popc(m);
+  }
+  __syncwarp();
+  int sh = 0;                                    // 2^sh lanes per output
+  while (sh < 5 && (total << (sh + 1)) <= 32) ++sh;
+  for (int base = 0; base < total; base += 32 >> sh) {
+    const int j = base + (lane >> sh);
+    double v = 0.0;
+    if (j < total) {
+      const int i = list[j] >> 5, l = list[j] & 31;
+      const double* xp = x + ((l >> 2) + 8 * (i >> 1)) * (ptrdiff_t)xa;
+      const double* yp = y + (2 * (l & 3) + (i & 1)) * (ptrdiff_t)yb;
+#pragma unroll 8
+      for (int k = lane & ((1 << sh) - 1); k < len; k += 1 << sh)
+        v = fma(xp[k * (ptrdiff_t)xk], yp[k * (ptrdiff_t)yk], v);
+    }
+    for (int o = (1 << sh) >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = at[i] - base;
+      const double w = __shfl_sync(0xffffffffu, v, (k << sh) & 31);
+      if (((need >> i) & 1u) && k >= 0 && k < (32 >> sh)) fix[i] = w;
+    }
+  }
+  __syncwarp();
+  return total;
+}
+__device__ __forceinline__ int redo(unsigned need, const double* x, int xa, int xk, const double* y, int yb, int yk,
+                                    int len, unsigned char* list, double (&out)[4]) {
+  double fix[4];
+  const int total = redo_list(need, x, xa, xk, y, yb, yk, len, list, fix);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    if ((need >> i) & 1u) out[i] = fix[i];
+  return total;
+}
+// V Y where nearly all outputs of 16 x 8 are weak: the digits are wasted, and a warp takes
+// its next tiles in plain FP64 before it tries again (elements over 10 decades, 35 columns to
+// 21: 803 us, and 998 us without this; with 80 for 112, log-normal(2) elements took 780 for 706).
+constexpr int WEAK_MANY = 112, WEAK_SKIP = 7;
 
 __device__ inline int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
 
@@ -361,8 +465,9 @@ __device__ __forceinline__ void row_digits(const double* tile, const int* b, int
 // acc = the 16 x 8 products of 16 rows of a tile with 8 coefficient columns
 template <int KT, int LDS_>
 __device__ __forceinline__ void rows_times_coeff(const double* tile, const Scales& sc, int set, const uint2* Bs, int g,
-                                                 int t, int lane, const int (&base)[2], Acc& acc) {
+                                                 int t, int lane, const int (&base)[2], Acc& acc, Mag& mag) {
   acc.clear();
+  mag.clear();
 #pragma unroll 1
   for (int kt = 0; kt < KT; ++kt) {
     unsigned a[NS][4];
@@ -379,11 +484,17 @@ __device__ __forceinline__ void rows_times_coeff(const double* tile, const Scale
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
       const uint2 b = Bs[((set * NS + q) * KT + kt) * 32 + lane];
+      if (q == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
 #pragma unroll
       for (int s = 0; s + q < NS; ++s) mma16(acc.c[acc_of(s, q)], a[s], b.x, b.y);
     }
   }
 }
+// Levels that make outputs 2 h, 2 h + 1 pass where they do not exist (columns 2 t, 2 t + 1 from q on).
+__device__ __forceinline__ unsigned no_cols(int t, int q) {
+  return (2 * t < q ? 0u : 31u) | (2 * t + 1 < q ? 0u : 31u << 16);
+}
+constexpr unsigned NO_ROW = 0x001f001fu;
 
 // ---------------------------------------------------------------------------
 // Out = P Y [- Xs diag(theta)], optional column norms.  A warp takes 16-row
@@ -460,6 +571,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   __shared__ Scales sc;
   __shared__ double wn[TS_W][8];
   __shared__ double part[8];
+  __shared__ unsigned char list[TS_W][128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   uint2* Bs = reinterpret_cast<uint2*>(smem_raw);
   double* buf = reinterpret_cast<double*>(smem_raw + off_tiles) + (size_t)warp * KT * 16 * TS_LD;
@@ -470,6 +582,8 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   coeff_frag_b<KT, TS_W * 32>(Y, ldy, p, r, sc, Bs, tid);
   const bool plain = sc.bad != 0;
   const int c0 = 2 * t;
+  int skip = 0;                                  // tiles to take in plain FP64
+  const unsigned pad = no_cols(t, r);
   double sq[2] = {0.0, 0.0}, th[2] = {0.0, 0.0};
   if (theta)
     for (int u = 0; u < 2; ++u) th[u] = c0 + u < r ? theta[c0 + u] : 0.0;
@@ -477,7 +591,8 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
     const int row0 = tile * TS_R, i0 = row0 + g, next = tile + stride;
     int base[2];
     const int set = row_scales<KT, TS_LD, 2>(buf, sc, g, t, base);
-    if (set < 0 || plain) {
+    if (set < 0 || plain || skip > 0) {
+      --skip;
       tall_plain(buf, row0, n, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, lane,
                  [&](int c, double v) { wn[warp][c] += v; });
       __syncwarp();
@@ -493,19 +608,33 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
         }
       }
       Acc acc;
-      rows_times_coeff<KT, TS_LD>(buf, sc, set, Bs, g, t, lane, base, acc);
-      __syncwarp();                              // every lane is done with the tile
-      if (next < ntiles) load_cols<TS_R, TS_LD, 32>(P, ldp, p, n, next * TS_R, vec, buf, lane);
-      cp_commit();
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      Mag mag;
+      rows_times_coeff<KT, TS_LD>(buf, sc, set, Bs, g, t, lane, base, acc, mag);
+      const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
+      auto finish = [&](int q, double o) {
         const int c = c0 + (q & 1), i = i0 + (q < 2 ? 0 : 8);
-        double o = times_pow2(acc.sum(q), base[q < 2 ? 0 : 1] + sc.F[set][c] - E_OUT);
         if (theta) o = fma(-th[q & 1], xs[q], o);
         if (c < r && i < n) {
           Out[(size_t)c * ldo + i] = o;
           if (norms2) sq[q & 1] = fma(o, o, sq[q & 1]);
         }
+      };
+      unsigned need = 0u;
+      if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+        need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
+        double fix[4];
+        if (redo_list(need, buf, 1, TS_LD, Y, ldy, 1, p, list[warp], fix) > WEAK_MANY) skip = WEAK_SKIP;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if ((need >> q) & 1u) finish(q, fix[q]);
+      }
+      __syncwarp();                              // every lane is done with the tile
+      if (next < ntiles) load_cols<TS_R, TS_LD, 32>(P, ldp, p, n, next * TS_R, vec, buf, lane);
+      cp_commit();
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const double o = times_pow2(acc.sum(q), base[q < 2 ? 0 : 1] + sc.F[set][c0 + (q & 1)] - E_OUT);
+        if (!((need >> q) & 1u)) finish(q, o);
       }
     }
     cp_wait<0>();
@@ -538,6 +667,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   constexpr int TS_W = tall_warps(KT);
   __shared__ Scales sc;
   __shared__ double part[64];
+  __shared__ unsigned char list[TS_W][128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int mt = (r + 15) / 16;
   uint4* As = reinterpret_cast<uint4*>(smem_raw);
@@ -550,16 +680,19 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   tall_start<KT>(n, P, ldp, p, Y, ldy, r, mt * 16, vec, buf, tile, ntiles, sc, tid);
   coeff_frag_a<KT, TS_W * 32>(Y, ldy, p, r, mt, sc, As, tid);
   const bool plain = sc.bad != 0;
+  int skip = 0;
   for (; tile < ntiles; tile += stride) {
     const int row0 = tile * TS_R, next = tile + stride;
     int base[2];
     const int set = row_scales<KT, TS_LD, 2>(buf, sc, g, t, base);
-    if (set < 0 || plain) {
+    if (set < 0 || plain || skip > 0) {
+      --skip;
       tall_plain(buf, row0, n, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, lane, [&](int c, double v) {
         if (norms2) slot[(c >> 4) * 64 + (c & 7) * 8 + ((c >> 3) & 1)] += v;
       });
     } else {
       const int* F = sc.F[set];
+      unsigned weak = 0u;                        // 4 bits per half of the rows and 16 columns
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         unsigned b[KT][NS][2];
@@ -581,16 +714,27 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
         for (int j = 0; j < mt; ++j) {
           const uint4* as = As + (size_t)(set * mt + j) * KT * NS * 32 + lane;
           Acc acc;
+          Mag mag;
           acc.clear();
+          mag.clear();
 #pragma unroll
           for (int kt = 0; kt < KT; ++kt)
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               const uint4 v = as[(kt * NS + s) * 32];
               const unsigned a[4] = {v.x, v.y, v.z, v.w};
+              if (s == 0) mag.add(v.x, v.y, v.z, v.w, b[kt][0][0], b[kt][0][1]);
 #pragma unroll
               for (int q = 0; s + q < NS; ++q) mma16(acc.c[acc_of(s, q)], a, b[kt][q][0], b[kt][q][1]);
             }
+          const unsigned pad = no_cols(t, n - row0 - 8 * h);   // (here the rows run along t)
+          const unsigned l0 = mag.levels(0) | pad | (j * 16 + g < r ? 0u : NO_ROW);
+          const unsigned l1 = mag.levels(1) | pad | (j * 16 + g + 8 < r ? 0u : NO_ROW);
+          unsigned need = 0u;
+          if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+            need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
+            weak |= need << (16 * h + 4 * j);
+          }
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
             const int c = j * 16 + g + 8 * u;
@@ -603,19 +747,40 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
                 if (i + 1 < n) o1 = fma(-th, Xs[(size_t)c * ldx + i + 1], o1);
               }
               double* o = Out + (size_t)c * ldo + i;
-              if (i + 1 >= n) {
-                o[0] = o0;
-                o1 = 0.0;
-              } else if (vec_out) {
+              const unsigned w = (need >> (2 * u)) & 3u;   // the weak ones of the two are left out
+              if (i + 1 >= n) o1 = 0.0;
+              if (w == 0u && i + 1 < n && vec_out) {
                 *reinterpret_cast<double2*>(o) = make_double2(o0, o1);
               } else {
-                o[0] = o0;
-                o[1] = o1;
+                if (!(w & 1u)) o[0] = o0;
+                if (!(w & 2u) && i + 1 < n) o[1] = o1;
               }
+              if (w & 1u) o0 = 0.0;
+              if (w & 2u) o1 = 0.0;
               if (norms2) slot[j * 64 + lane * 2 + u] += fma(o0, o0, o1 * o1);
             }
           }
         }
+      }
+      if (__any_sync(0xffffffffu, weak)) {
+        int most = 0;
+        for (int h = 0; h < 2; ++h)
+          for (int j = 0; j < mt; ++j) {
+            const unsigned need = (weak >> (16 * h + 4 * j)) & 15u;
+            if (!__any_sync(0xffffffffu, need)) continue;
+            double fix[4];
+            most = max(most, redo_list(need, Y + (size_t)j * 16 * ldy, ldy, 1, buf + 8 * h, 1, TS_LD, p, list[warp], fix));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              if (!((need >> q) & 1u)) continue;
+              const int c = j * 16 + g + 8 * (q >> 1), i = row0 + 8 * h + 2 * t + (q & 1);
+              double o = fix[q];
+              if (theta) o = fma(-theta[c], Xs[(size_t)c * ldx + i], o);
+              Out[(size_t)c * ldo + i] = o;
+              if (norms2) slot[j * 64 + lane * 2 + (q >> 1)] += o * o;
+            }
+          }
+        if (most > WEAK_MANY) skip = WEAK_SKIP;
       }
     }
     __syncwarp();                                // every lane is done with the tile
@@ -669,6 +834,16 @@ __device__ __forceinline__ int col_scale(const double* col, int t, bool& ok) {
   return e;
 }
 
+// For a pair of outputs (halves) of a chunk with the scales e and the levels l of its sums of
+// moduli: top = the larger of it and e + l.  The chunk's digits will do where e + MAG_MIN <= top: they are
+// then off by no more than the chain against the largest sum so far.  (A CTA takes a second
+// tile only when there are more than 2 x 152, so that the errors of its chunks, each within (K + 4)
+// 2^-52 of that sum, stay within n / 64 + 64 such parts of all.)
+__device__ __forceinline__ unsigned raise(unsigned e, unsigned l, unsigned& top) {
+  top = __vmaxu2(top, e + l);
+  return e + MAG_MIN;
+}
+
 template <int KT>
 __global__ void __launch_bounds__(CS_W * 32, 2)
     k_cgs_split(int n, Basis<double> P, double* __restrict__ Tb, int ldt, int q, const double* __restrict__ Gsub,
@@ -677,6 +852,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
   constexpr int CH = KT >= 3 ? 2 : KT == 2 ? 4 : 8, RC = CS_R / CH, KS = RC / 16;   // chunks of RC rows, KS steps each
   __shared__ Scales sc;
   __shared__ int te[CH][8], tok[CH];
+  __shared__ unsigned char list[CS_W][128];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int p = P.cols();
   uint2* Bs = reinterpret_cast<uint2*>(smem_raw);                    // Gsub, both sets of scales
@@ -688,6 +864,10 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
   __syncthreads();
   const int ntiles = (n + CS_R - 1) / CS_R;
   double gacc[4] = {0.0, 0.0, 0.0, 0.0}, tacc[2] = {0.0, 0.0};
+  // level of the largest sum of moduli among the chunks so far, two outputs to a register:
+  // a chunk that lies wholly below it needs no better than the digits give
+  unsigned gtop[2] = {0u, 0u}, ttop = 0u;
+  const unsigned pad = no_cols(t, q);
   const int ch = warp / KT, m = warp % KT;       // this warp's chunk and columns of P^T T (none when ch >= CH)
   const int tch = KT == 3 ? (warp >= 6 ? warp - 6 : -1) : (m == 0 ? ch : -1);   // its chunk of T^T T
   bool first = true;
@@ -722,13 +902,28 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
         }
       } else {
         Acc acc;
-        rows_times_coeff<KT, CS_LD>(cur, sc, set, Bs, g, t, lane, base, acc);
+        Mag mag;
+        rows_times_coeff<KT, CS_LD>(cur, sc, set, Bs, g, t, lane, base, acc, mag);
+        const int i0 = row0 + 16 * warp + g;       // (rows past n are zero)
+        const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
+        double out[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int c = 2 * t + (i & 1);
-          tw[c * CS_LD + g + (i < 2 ? 0 : 8)] -=
-              times_pow2(acc.sum(i), base[i < 2 ? 0 : 1] + sc.F[set][c] - E_OUT);
+        for (int i = 0; i < 4; ++i)
+          out[i] = times_pow2(acc.sum(i), base[i < 2 ? 0 : 1] + sc.F[set][2 * t + (i & 1)] - E_OUT);
+        if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+          unsigned need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
+          // the digits' error, below 2^5 of the sum's last place, is no matter where it is below
+          // half an ulp of T (their last place is 2^(base + F - E_OUT))
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int c = 2 * t + (i & 1);
+            if (expo(tw[c * CS_LD + g + (i < 2 ? 0 : 8)]) >= base[i < 2 ? 0 : 1] + sc.F[set][c] - E_OUT + 5 + 1023 + 53)
+              need &= ~(1u << i);
+          }
+          if (__any_sync(0xffffffffu, need)) redo(need, cur, 1, CS_LD, Gsub, p, 1, p, list[warp], out);
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) tw[(2 * t + (i & 1)) * CS_LD + g + (i < 2 ? 0 : 8)] -= out[i];
       }
       __syncwarp();
       for (int e = lane; e < q * 16; e += 32) {
@@ -760,7 +955,9 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
         const int e0 = col_scale<RC>(x0, t, ok), e1 = col_scale<RC>(x0 + 8 * CS_LD, t, ok);
         if (__all_sync(0xffffffffu, ok)) {
           Acc acc;
+          Mag mag;
           acc.clear();
+          mag.clear();
 #pragma unroll 1
           for (int ks = 0; ks < KS; ++ks) {
             unsigned a[NS][4];
@@ -780,13 +977,24 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
               const uint2 b = Td[((ch * KS + ks) * NS + k) * 32 + lane];
+              if (k == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
 #pragma unroll
               for (int s = 0; s + k < NS; ++s) mma16(acc.c[acc_of(s, k)], a[s], b.x, b.y);
             }
           }
+          const int s0 = te[ch][2 * t], s1 = te[ch][2 * t + 1];
+          const unsigned s01 = (unsigned)s0 | (unsigned)s1 << 16;
+          const unsigned w0 = raise(e0 * 0x10001u + s01, mag.levels(0) | pad | (16 * m + g < p ? 0u : NO_ROW), gtop[0]);
+          const unsigned w1 = raise(e1 * 0x10001u + s01, mag.levels(1) | pad | (16 * m + g + 8 < p ? 0u : NO_ROW), gtop[1]);
+          double out[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            gacc[i] += times_pow2(acc.sum(i), (i < 2 ? e0 : e1) + te[ch][2 * t + (i & 1)] - E_OUT);
+            out[i] = times_pow2(acc.sum(i), (i < 2 ? e0 : e1) + (i & 1 ? s1 : s0) - E_OUT);
+          if (any_less2(gtop[0], w0) || any_less2(gtop[1], w1))
+            redo(less2(gtop[0], w0) | less2(gtop[1], w1) << 2, Ps + 16 * m * CS_LD + ch * RC, CS_LD, 1, Ts + ch * RC,
+                 CS_LD, 1, RC, list[warp], out);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) gacc[i] += out[i];
         } else {
 #pragma unroll 1
           for (int i = 0; i < 4; ++i) {
@@ -804,7 +1012,9 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
       if (Tout && tch >= 0 && tch < CH) {
         if (tok[tch]) {
           Acc acc;
+          Mag mag;
           acc.clear();
+          mag.clear();
 #pragma unroll 1
           for (int ks = 0; ks < KS; ++ks) {
             uint2 b[NS];
@@ -813,12 +1023,18 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               const unsigned a[4] = {b[s].x, 0u, b[s].y, 0u};
+              if (s == 0) mag.add(b[0].x, 0u, b[0].y, 0u, b[0].x, b[0].y);
 #pragma unroll
               for (int k = 0; s + k < NS; ++k) mma16(acc.c[acc_of(s, k)], a, b[k].x, b[k].y);
             }
           }
-#pragma unroll
-          for (int i = 0; i < 2; ++i) tacc[i] += times_pow2(acc.sum(i), te[tch][g] + te[tch][2 * t + i] - E_OUT);
+          const int e = te[tch][g], s0 = e + te[tch][2 * t], s1 = e + te[tch][2 * t + 1];
+          const unsigned w = raise((unsigned)s0 | (unsigned)s1 << 16, mag.levels(0) | pad | (g < q ? 0u : NO_ROW), ttop);
+          double out[4] = {times_pow2(acc.sum(0), s0 - E_OUT), times_pow2(acc.sum(1), s1 - E_OUT), 0.0, 0.0};
+          if (any_less2(ttop, w))
+            redo(less2(ttop, w), Ts + tch * RC, CS_LD, 1, Ts + tch * RC, CS_LD, 1, RC, list[warp], out);
+          tacc[0] += out[0];
+          tacc[1] += out[1];
         } else {
           for (int i = 0; i < 2; ++i) {
             const double *x = Ts + g * CS_LD + tch * RC, *y = Ts + (2 * t + i) * CS_LD + tch * RC;

@@ -205,3 +205,75 @@ def test_fp32_streaming(h, n, p, r):
     if r <= p:
         out, _ = _tall(h, P, Y, fp32=True, inplace=True)
         assert np.all(np.abs(out - P64 @ Y32) <= (p + 2) * e32 * (np.abs(P64) @ np.abs(Y32)))
+
+
+def _peaks(rng, n, p, peak, kind):
+    """Rows whose magnitudes differ element by element, not by rows or columns."""
+    P = rng.standard_normal((n, p))
+    if kind == "one":                                       # one element of each row
+        P[np.arange(n), np.arange(n) % p] *= peak
+    elif kind == "few":                                     # one element in some tiles
+        rows = np.arange(5, n, 37)
+        P[rows, rows % p] = peak
+    else:                                                   # spread over all decades
+        P *= peak ** rng.uniform(-1, 1, (n, p))
+    return P
+
+
+@pytest.mark.parametrize("p,r", [(9, 4), (35, 21), (20, 8), (60, 30)])
+@pytest.mark.parametrize("peak", [1e3, 1e6, 1e10, 1e25])
+@pytest.mark.parametrize("kind", ["one", "few", "spread"])
+def test_tall_peaks_inside_a_row(h, p, r, peak, kind):
+    """An output whose terms are far below (row maximum) x (coefficient maximum) is as
+    accurate as a chain of multiply-adds: within (p + 4) eps of its sum of moduli."""
+    rng = np.random.default_rng(p)
+    n = 1000
+    P = _peaks(rng, n, p, peak, kind)
+    zero = rng.standard_normal((p, r))
+    zero[:: 3] = 0.0                                        # some peaks meet a zero coefficient
+    for Y in (zero, np.eye(p)[:, :r], np.eye(p)[:, :r] + 1e-3 * rng.standard_normal((p, r))):
+        out, _ = _tall(h, P, Y)
+        S = np.abs(P) @ np.abs(Y)
+        assert np.all(np.abs(out - _mm(P, Y)) <= (p + 4) * EPS * S)
+
+
+def test_tall_peak_with_a_zero_coefficient(h):
+    P = np.ones((600, 11))
+    P[300, 0] = 1e25
+    Y = np.ones((11, 3))
+    Y[0] = 0.0
+    out, _ = _tall(h, P, Y)
+    assert np.all(out == 10.0)
+
+
+@pytest.mark.parametrize("n,p,q", [(4000, 12, 5), (4001, 35, 8), (9000, 64, 3), (80001, 35, 6)])
+@pytest.mark.parametrize("peak", [1e3, 1e8, 1e25])
+@pytest.mark.parametrize("kind", ["one", "few", "spread"])
+def test_block_cgs_peaks_inside_a_row_and_a_column(h, n, p, q, peak, kind):
+    """The same for T - P Gsub (beside |T|), and for P^T T and T^T T within n / 64 + 64 eps
+    of the sums of moduli: single elements of T where P is zero, peaks of P where T is small."""
+    rng = np.random.default_rng(n + q)
+    P = _peaks(rng, n, p, peak, kind)
+    T = rng.standard_normal((n, q)) if kind != "spread" else _peaks(rng, n, q, peak, kind)
+    rows = np.arange(11, n, 64)
+    P[rows] = 0.0
+    T[rows, rows % q] = peak
+    G = rng.standard_normal((p, q))
+    G[:: 3] = 0.0
+    Pd, Gd = _dev(P, n), torch.from_numpy(np.ascontiguousarray(G.T)).cuda()
+    for sub in (False, True):
+        Td = _dev(T, n)
+        Go = torch.zeros(p * q, dtype=torch.float64, device="cuda")
+        To = torch.zeros(q * q, dtype=torch.float64, device="cuda")
+        native.phsvds_block_cgs(h, n, None, n, 0, Td, n, q, Gsub=Gd if sub else None, Gout=Go, Tout=To, P2=Pd, ld2=n,
+                                p2=p)
+        native.phsvds_sync(h)
+        T2 = Td.cpu().numpy().T
+        if sub:
+            assert np.all(np.abs(T2 - (T.astype(L) - _mm(P, G))) <= (p + 4) * EPS * (np.abs(T) + np.abs(P) @ np.abs(G)))
+        else:
+            assert np.array_equal(T2, T)
+        for buf, A in ((Go, P), (To, T2)):
+            got = buf.cpu().numpy().reshape(q, -1).T
+            lim = (n / 64 + 64) * EPS * (np.abs(A).T @ np.abs(T2))
+            assert np.all(np.abs(got - _mm(A.T, T2)) <= lim)
