@@ -419,10 +419,14 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
       } else if (fabs(m) <= E_SMALL * fabs(gap)) {
         if (m != 0.0) {
           // 1 / gap by one Newton step from FP32 (the quotient only has to be
-          // good to a share of itself)
+          // good to a share of itself), where FP32 holds the gap and its reciprocal
           const double gs = gap * down;
-          const double y = (double)__frcp_rn((float)gs);
-          k = m * down * (y * fma(-gs, y, 2.0));
+          if (fabs(gs) > 1e-37) {
+            const double y = (double)__frcp_rn((float)gs);
+            k = m * down * (y * fma(-gs, y, 2.0));
+          } else {
+            k = m / gap;
+          }
           if (fabs(k) > E_ANGLE && fabs(m) <= noise) k = 0.0;
         }
       } else if ((sm.tgt[r] || sm.tgt[c]) && fabs(m) > noise) {

@@ -4,6 +4,7 @@ columns, up to 64), both targets, and multiple eigenvalues, against the dense
 SVD."""
 import numpy as np
 import pytest
+import scipy.sparse as sp
 
 from paper_1408_5535_gb300 import native, synth
 from tests.gpu_util import need_gpu
@@ -59,3 +60,23 @@ def test_multiple_singular_values_keep_the_basis_orthonormal(h, mat, start):
     sig, U, V, _, _, _ = native.phsvds_solve(h, A.m, A.n, A.row_ptr, A.col, A.val, 8, native.SMALLEST, 1e-13, opts=o)
     assert np.all(np.abs(sig - np.sort(sigma)[:8]) <= 1e-10)
     assert np.max(np.abs(V.T @ V - np.eye(8))) <= 1e-11
+
+
+@pytest.mark.parametrize("scale,tiny", [(1.0, 1e-20), (1e3, 1e-60), (1e10, 1e-160)])
+def test_gaps_below_the_range_of_fp32(h, scale, tiny):
+    """Two columns of A that meet no other and are smaller by 20 to 170 decades: the gap of
+    their Ritz values has no reciprocal in FP32, and at last none after scaling in FP64."""
+    n, m = 100, 160
+    rng = np.random.default_rng(3)
+    D = np.zeros((m, n))
+    D[:150, :98] = scale * rng.standard_normal((150, 98)) * (rng.random((150, 98)) < 0.2)
+    D[150, 98], D[151, 98], D[151, 99] = tiny, 1e-2 * tiny, 3 * tiny
+    S = sp.csr_matrix(D)
+    x0 = np.zeros((n, 6))
+    x0[98, 0] = x0[99, 1] = 1.0
+    x0[:98, 2:] = rng.standard_normal((98, 4))
+    o = native.default_opts(block_size=2)
+    sig = native.phsvds_solve(h, m, n, S.indptr.astype(np.int64), S.indices.astype(np.int32), S.data, 3,
+                              native.LARGEST, 1e-13, opts=o, init_V=x0)[0]
+    ref = np.linalg.svd(D, compute_uv=False)[:3]
+    assert np.all(np.abs(sig - ref) <= 1e-10 * ref)
