@@ -23,9 +23,14 @@
 //    by columns, each CTA its own (the products are independent of one another,
 //    where FP64 Jacobi rounds depend on the one before).  Two or three steps
 //    take the FP32 vectors to FP64;
-//  * a pair whose m_ij is not small against its gap is rotated first, if one of
-//    the two is a target; other such pairs only span the restart space and are
-//    left as they are.
+//  * where a target's m_ij is not small against its gap, the targets and all that is
+//    coupled to them in this way, directly or through others, are rotated first: X
+//    is made orthonormal (to first order, so that the matrix of the m_ij is X^T H X),
+//    then classical Jacobi until every m_ij of these rows is below E_ROT of its gap.
+//    Rotating X^T H X of an X that is orthonormal to FP32 only, or the targets alone,
+//    ends with the couplings of a cluster as they were: lambda G_ij outweighs its
+//    gaps, and the first-order steps go through the pairs left out.  Other such pairs
+//    only span the restart space and are left as they are.
 // FP64 instructions hold an SM's pipe for 16 clocks a warp, so what is not a
 // product (maxima, ranks, angles) runs on integers or in FP32.
 // Measured: 75 us at j = 28 (of 145,000 clocks 74,000 in 108 Jacobi rounds, 54,000
@@ -54,6 +59,11 @@ constexpr int EMAT = EJ * EL;
 constexpr int FL = EJ + 14, FMAT = EJ * FL;
 constexpr int E_STEPS = 8;             // refinement steps at most (two or three are usual)
 constexpr double E_SMALL = 0.02;       // m_ij / gap up to which a pair is refined; above, rotated
+// ... down to this: in a cluster the second-order terms add up over its members and the ratios
+// of its gaps (emulated, 14 values within 1e-4 and the couplings that FP32 leaves: from 0.02
+// the steps run out in a quarter of the cases, from here in none; 93 rotations, and 4 steps for 7)
+constexpr double E_ROT = 3e-4;
+constexpr int E_MOST = 8 * EJ;         // rotations at most
 // Largest |E_ij| after which the update has reached FP64: it leaves X^T X = I + O(j
 // E^2), and a basis transformed by less orthogonal coefficients drifts over the
 // restarts.
@@ -73,6 +83,8 @@ struct EigSmem {
   unsigned redu[EW];
   int rank[EJ];
   int sel;
+  double wbest[EW];
+  int wat[EW];
   unsigned char tgt[EJ];
 };
 
@@ -347,6 +359,7 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
   // square of the orthogonality: such a pair is left as it is.
   const double noise = 4.0 * 2.220446049250313e-16 * mx;
   bool last = false;                               // this step only makes X orthonormal
+  bool stuck = false;                              // the steps ran out
   int step = 0, turned = 0;
   float before = INFINITY;
   while (true) {
@@ -459,35 +472,75 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
 #pragma unroll
     for (int k = 0; k < EC; ++k) e = fmaxf(e, sm.wmax[k]);
     if (isinf(e) && turned < 4 && step < E_STEPS) {
-      // ---- rotate the flagged pairs, the largest |B_ij| first, in every CTA alike
+      // ---- rotate, the largest |m_ij| first, in every CTA alike
       ++turned;
-      for (int i = warp; i < ncol; i += EW)
-        for (int r = lane; r < j; r += 32)
-          for (int k = 0; k < EC; ++k) peer[k]->B[r + (cr + i * EC) * EL] = sm.Bc[i][r];
-      cl.sync();
-      for (int n = 0; n < 2 * EJ; ++n) {
-        if (warp == 0) {
-          double best = 0.0;
-          int at = -1;
-          for (int t = 0; t < j; ++t) {
-            if (!sm.tgt[t]) continue;
-            for (int r = lane; r < j; r += 32) {
-              const double b = fabs(sm.B[r + t * EL]), gap = fabs(sm.B[t + t * EL] - sm.B[r + r * EL]);
-              if (r != t && b > noise && b > E_SMALL * gap && b > best) {
-                best = b;
-                at = r + t * 64;
-              }
-            }
-          }
+      for (int q = tid; q < ncol * j; q += ET) {
+        const int i = q / j, r = q - i * j, c = cr + i * EC;
+        const double gr = sm.Gc[i][r], lr = sm.lam[r], lc = sm.lam[c];
+        const double m = r == c ? lc : fma(-0.5 * (lr + lc), gr, sm.Bc[i][r]);
+        sm.Ec[i][r] = r == c ? 0.5 * (1.0 - gr) : -0.5 * gr;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) {
-            const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oa = __shfl_xor_sync(0xffffffffu, at, o);
-            if (ob > best || (ob == best && oa > at)) {
-              best = ob;
-              at = oa;
+        for (int k = 0; k < EC; ++k) peer[k]->B[r + c * EL] = m;
+      }
+      __syncthreads();
+      for (int q = tid; q < ncol * j; q += ET) {
+        const int i = q / j, r = q - i * j, at = r + (cr + i * EC) * EL;
+        const double v = X[at] + dot_col(X + r, EL, sm.Ec[i], j);
+#pragma unroll
+        for (int k = 0; k < EC; ++k) peer[k]->X[xb ^ 1][at] = v;
+      }
+      cl.sync();
+      xb ^= 1;
+      X = sm.X[xb];
+      auto coupled = [&](int r, int t, double b, double tau) {
+        return b > noise && b > tau * fabs(sm.B[t + t * EL] - sm.B[r + r * EL]);
+      };
+      // what is coupled to the targets joins them
+      while (true) {
+        unsigned hits = 0u;                        // bit i: column warp + i EW is coupled to one of them
+        for (int t = warp, i = 0; t < j; t += EW, ++i) {
+          bool hit = false;
+          for (int r = lane; r < j && !sm.tgt[t]; r += 32)
+            hit = hit || (sm.tgt[r] && coupled(r, t, fabs(sm.B[r + t * EL]), E_SMALL));
+          if (__any_sync(0xffffffffu, hit)) hits |= 1u << i;
+        }
+        if (!__syncthreads_or(hits != 0u)) break;
+        if (lane == 0)
+          for (int i = 0; i < EJ / EW; ++i)
+            if ((hits >> i) & 1u) sm.tgt[warp + i * EW] = 1;
+        __syncthreads();
+      }
+      for (int n = 0; n < E_MOST; ++n) {
+        double best = 0.0;
+        int at = -1;
+        for (int t = warp; t < j; t += EW) {
+          if (!sm.tgt[t]) continue;
+          for (int r = lane; r < j; r += 32) {
+            const double b = fabs(sm.B[r + t * EL]);
+            if (r != t && b > best && coupled(r, t, b, E_ROT)) {
+              best = b;
+              at = r + t * 64;
             }
           }
+        }
+        auto larger = [&](double ob, int oa) {
+          if (ob > best || (ob == best && oa > at)) {
+            best = ob;
+            at = oa;
+          }
+        };
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+          larger(ob, __shfl_xor_sync(0xffffffffu, at, o));
+        }
+        if (lane == 0) {
+          sm.wbest[warp] = best;
+          sm.wat[warp] = at;
+        }
+        __syncthreads();
+        if (warp == 0) {
+          for (int w = 1; w < EW; ++w) larger(sm.wbest[w], sm.wat[w]);
           if (at >= 0) {
             // the angle in FP32 (what it leaves is refined), c and s orthonormal
             // in FP64: c = x^(-1/2), x = 1 + t^2, by a Halley step
@@ -506,7 +559,7 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
           if (lane == 0) sm.sel = at;
         }
         __syncthreads();
-        const int at = sm.sel;
+        at = sm.sel;
         if (at < 0) break;
         const int p = min(at & 63, at >> 6), q = max(at & 63, at >> 6);
         const double c = sm.rot[0], s = sm.rot[1];
@@ -541,7 +594,9 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
     // done, or on the rounding floor of a pair that is nearly one; what a last large
     // rotation has cost X is mended by one more step
     if (last) break;
-    if (!(e > E_DONE) || (e < 1e-7f && e > 0.1f * before) || step >= E_STEPS) {
+    const bool done = !(e > E_DONE) || (e < 1e-7f && e > 0.1f * before);
+    if (done || step >= E_STEPS) {
+      stuck = !done;
       if (!(e > E_ANGLE)) break;
       last = true;
     }
@@ -566,6 +621,7 @@ __global__ void __cluster_dims__(EC, 1, 1) __launch_bounds__(ET, 1) k_eig_step(E
       g.counters[1] = rots;
       g.counters[2] = step;
       g.counters[3] = turned;
+      g.counters[4] = stuck;
     }
   }
 }

@@ -234,7 +234,9 @@ void jacobi_eig32_ld(cudaStream_t s, int j, const double* H, int ldh, double* Sf
 // with S^T H S diagonal to FP64 in the rows of the ntarget smallest (tmode 0) or
 // largest (1) eigenvalues and to FP32 or better elsewhere; theta = the diagonal, order =
 // its ranking, Scols / thcols = the nt first in that order.  counters: FP32
-// sweeps, rotations, refinement steps, steps that rotated.  1 <= j <= 64.
+// sweeps, rotations, refinement steps, steps that rotated, and whether the steps ran
+// out before the target rows were diagonal (S is orthonormal then, no more).
+// 1 <= j <= 64.
 // norms[0 .. nt) is zeroed for the sums that follow; with *skip != 0 that is all.
 void eig_step(cudaStream_t s, int j, const double* H, double* S, int ld, bool ident, int ntarget, int tmode, int nt,
               double* theta, int* order, double* Scols, double* thcols, double* norms, int* counters, const int* skip);

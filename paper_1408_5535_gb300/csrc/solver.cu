@@ -740,6 +740,7 @@ struct Stage1Out {
   int64_t jac_sweeps = 0, jac_rot = 0, jac_calls = 0, jac_dim = 0;
   int fell_back = 0;
   int64_t fell_back_at = 0, recorded = 0, stag_locks = 0;
+  int64_t eig_short = 0;   // projected solves whose refinement ran out of steps
 };
 
 // Device state of the learned correction (PHSVDS_PREC_LEARNED) for one solve.
@@ -1144,7 +1145,8 @@ struct Stage1 {
       s_ident = false;
       out.iters++;
       if (*h.at<int>(968)) throw PhError{PHSVDS_ERR_NAN, "stage 1: corrupted ordering of the Ritz values"};
-      if (mixed_eig) {  // FP32 pass + FP64 clean-up
+      if (one_eig && *h.at<int>(992)) ++out.eig_short;
+      if (mixed_eig) {  // FP32 pass and what follows it in FP64
         out.jac_sweeps += *h.at<int>(976) + *h.at<int>(984);
         out.jac_rot += *h.at<int>(980) + *h.at<int>(988);
       } else {
@@ -1198,9 +1200,9 @@ struct Stage1 {
       }
       if (!unconv.empty()) history.push_back(std::sqrt(std::max(hn[unconv[0]], 0.0)));
       if (trace_on())
-        fprintf(stderr, "s1[%d] it=%lld j=%d nlock=%d th0=%.17g rn0=%.6e thmax=%.6e nconv=%d\n", (int)sizeof(T),
-                (long long)out.iters, j, nlock, thv[0], std::sqrt(std::max(hn[0], 0.0)), out.theta_max,
-                (int)conv.size());
+        fprintf(stderr, "s1[%d] it=%lld j=%d nlock=%d th0=%.17g rn0=%.6e thmax=%.6e nconv=%d eig short=%lld\n",
+                (int)sizeof(T), (long long)out.iters, j, nlock, thv[0], std::sqrt(std::max(hn[0], 0.0)), out.theta_max,
+                (int)conv.size(), (long long)out.eig_short);
       if (rec_r && rec_every > 0 && out.recorded < rec_max && out.iters % rec_every == 0 && nt > 0) {
         if constexpr (sizeof(T) == 8) {
           CUCHK(cudaMemcpyAsync(rec_r + (size_t)out.recorded * n, Rr, sizeof(double) * n, cudaMemcpyDeviceToHost, s));
