@@ -83,31 +83,41 @@ inline cudaLaunchConfig_t cluster_config(A* at, int nc, int threads, size_t smem
 }
 
 // CTAs of the kernel's cluster on this device: 16 where it can be placed with smem
-// bytes, else 8.  Sets the kernel's attributes (up to smem_max bytes) at first use.
+// bytes, else 8, else 0 (the general form has to run).  Sets the kernel's attributes (up
+// to smem_max bytes) at first use.
 template <typename K>
 int cluster_size(K kernel, int threads, size_t smem, size_t smem_max, std::atomic<int> (&known)[64]) {
+  constexpr int NONE = -1;
   int dev = 0;
-  cudaGetDevice(&dev);
-  int nc = known[dev & 63].load(std::memory_order_acquire);
-  if (nc) return nc;
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  nc = 8;
-  cudaLaunchAttribute at[1];
-  const cudaLaunchConfig_t cfg = cluster_config(at, 16, threads, smem, nullptr);
-  int fit = 0;
-  if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess && fit > 0) nc = 16;
-  cudaGetLastError();
-  known[dev & 63].store(nc, std::memory_order_release);
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const int was = known[dev & 63].load(std::memory_order_acquire);
+  if (was) return was == NONE ? 0 : was;
+  if (cudaPeekAtLastError() != cudaSuccess) return 0;   // an earlier error is its caller's to see
+  int nc = 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) == cudaSuccess &&
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+    for (int c = 16; c >= 8 && nc == 0; c /= 2) {
+      cudaLaunchAttribute at[1];
+      const cudaLaunchConfig_t cfg = cluster_config(at, c, threads, smem, nullptr);
+      int fit = 0;
+      if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) == cudaSuccess && fit > 0) nc = c;
+    }
+  if (nc < 16) cudaGetLastError();
+  known[dev & 63].store(nc ? nc : NONE, std::memory_order_release);
   return nc;
 }
 
+// False: the launch was refused, nothing runs.
 template <typename K, typename G>
-void launch_cluster(K kernel, int nc, int threads, size_t smem, cudaStream_t s, const G& args) {
+bool launch_cluster(K kernel, int nc, int threads, size_t smem, cudaStream_t s, const G& args) {
   cudaLaunchAttribute at[1];
   const cudaLaunchConfig_t cfg = cluster_config(at, nc, threads, smem, s);
-  cudaLaunchKernelEx(&cfg, kernel, args);
+  if (cudaLaunchKernelEx(&cfg, kernel, args) != cudaSuccess) {
+    cudaGetLastError();                            // (an error that lasts is met again by the general form)
+    return false;
+  }
   count_launch();
+  return true;
 }
 
 }  // namespace ph

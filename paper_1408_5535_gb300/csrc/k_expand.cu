@@ -284,12 +284,12 @@ bool go(cudaStream_t s, ExArgs g) {
   constexpr size_t SMEM_MAX = 200 * 1024;
   g.cap = ((std::max(g.nlock + g.j, g.j + g.nb) + Q) * Q + 1) & ~1;
   g.nc = cluster_size(k_expand_cluster<T, Q>, XT, SMEM_MAX, SMEM_MAX, known);
+  if (g.nc == 0) return false;
   if (g.n <= 2048) g.nc = 8;                       // as fast as 16 at n = 1000 (143 us per iteration both)
   g.rows = ((g.n + g.nc - 1) / g.nc + 1) & ~1;
   const size_t smem = expand_smem(g.nc, g.cap, Q, g.rows, sizeof(T));
   if (smem > SMEM_MAX) return false;
-  launch_cluster(k_expand_cluster<T, Q>, g.nc, XT, smem, s, g);
-  return true;
+  return launch_cluster(k_expand_cluster<T, Q>, g.nc, XT, smem, s, g);
 }
 
 }  // namespace

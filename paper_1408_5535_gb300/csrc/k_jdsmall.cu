@@ -342,10 +342,10 @@ int cluster_ctas() {
 }
 
 template <typename T, int Q>
-void go(cudaStream_t s, JdArgs g) {
+bool go(cudaStream_t s, JdArgs g) {
   // (a barrier of 8 costs less than short vectors gain from 16)
   g.nc = std::min(cluster_ctas<T, Q>(), g.n <= 4 * JT ? 8 : 16);
-  launch_cluster(k_jd_cluster<T, Q>, g.nc, JT, sizeof(JdSmem<T>), s, g);
+  return g.nc && launch_cluster(k_jd_cluster<T, Q>, g.nc, JT, sizeof(JdSmem<T>), s, g);
 }
 
 }  // namespace
@@ -393,12 +393,11 @@ bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>&
   g.done = done;
   g.tol = tol;
   switch (Q) {
-    case 1: go<T, 1>(s, g); break;
-    case 2: go<T, 2>(s, g); break;
-    case 4: go<T, 4>(s, g); break;
-    default: go<T, 8>(s, g); break;
+    case 1: return go<T, 1>(s, g);
+    case 2: return go<T, 2>(s, g);
+    case 4: return go<T, 4>(s, g);
+    default: return go<T, 8>(s, g);
   }
-  return true;
 }
 template bool jd_solve_small<float>(cudaStream_t, const SparseView<float>&, const SparseView<float>&, int, int, bool,
                                     const float*, const float*, const float*, const double*, float*, float*, float*,

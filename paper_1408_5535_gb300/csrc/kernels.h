@@ -302,8 +302,8 @@ void s2_step(cudaStream_t s, int64_t N, int nq, const double* Bv, double* v, con
              const double* x, const double* Bx, double* tbest, double* acc, double* sc, double eta_tol, int patience,
              int maxit);
 // All steps of the block's solve in one launch of one cluster (k_jdsmall.cu), when
-// a step moves at most JD_SMALL_BYTES (false otherwise: nothing launched; the
-// measurements of both sides are in k_jdsmall.cu).
+// a step moves at most JD_SMALL_BYTES (false otherwise, and where the cluster cannot
+// be launched: nothing runs; the measurements of both sides are in k_jdsmall.cu).
 // After jd_init, with the same vectors: cv n x q, xrm n x width and z m x width
 // scratch (width q padded to 1, 2, 4 or 8); X null in the scaled form; done
 // (device int): the steps taken.
@@ -317,7 +317,8 @@ bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>&
 // the new rows and columns of Ht and S (unit), zero rows j.. of the nsp columns of
 // sprev.  flags[c], flags[nb]: as chol_factor, *bad = flags[nb]; when set, only Tb
 // was written besides.
-// xrm n x 8 and z m x width scratch.  False (nothing launched): too large.
+// xrm n x 8 and z m x width scratch.  False (nothing runs): too large, or the cluster
+// cannot be launched.
 template <typename T>
 bool expand_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& At, int nb, int nlock, int j, int nsp,
                   const T* Xl, T* V, T* W, T* Tb, T* xrm, T* z, double* Ht, double* S, double* sprev, int ldh,
