@@ -123,6 +123,11 @@ struct Host {
   template <typename T> T* at(size_t off_bytes) { return reinterpret_cast<T*>(base + off_bytes); }
 };
 
+// Its areas that reach past the few bytes of a readback, and the one that must outlast others.
+constexpr size_t HOST_BYTES = 1 << 16, HOST_NORM = 1024, HOST_STEP = 40960;
+static_assert(HOST_NORM + sizeof(double) * LD * LD <= HOST_STEP && HOST_STEP + sizeof(int) <= HOST_BYTES,
+              "the pending step count would share its bytes");
+
 // ---- instrumentation (per host thread)
 static thread_local int64_t g_launch_count = 0;
 void count_launch() { ++g_launch_count; }
@@ -627,7 +632,7 @@ struct InnerJD : InnerSolver {
     sc = pool.get<double>(JD_NSCALAR * 8);
     g1 = pool.get<double>(8 * 64);
     nstep = pool.get<int>(1);
-    hstep = Host(c).at<int>(20480);   // bytes [20480, 20484), nobody else's
+    hstep = Host(c).at<int>(HOST_STEP);   // read later than the other readbacks: nobody else's bytes
     graphs.enabled = use_graphs;
   }
   // the caller's vectors into the solve's precision, and the result back
@@ -2105,7 +2110,7 @@ static double lanczos_normC(phsvds_ctx* ctx, Pool& pool, const COp<double>& op, 
     scal(s, n, 1.0 / beta, nullptr, v1);
   }
   const int jl = (int)al.size();
-  double* hT = h.at<double>(1024);   // bytes [1024, 1024 + 8 LD^2)
+  double* hT = h.at<double>(HOST_NORM);   // bytes [HOST_NORM, HOST_NORM + 8 LD^2)
   for (int c = 0; c < jl; ++c)
     for (int r = 0; r < jl; ++r)
       hT[r + c * jl] = r == c ? al[c] : (r == c + 1 || c == r + 1) ? be[std::min(r, c)] : 0.0;
@@ -2796,7 +2801,7 @@ phsvds_status phsvds_create(phsvds_handle* out, int device, void* stream) {
     }
     c->own_stream = true;
   }
-  c->host_bytes = 1 << 16;
+  c->host_bytes = ph::HOST_BYTES;
   if (cudaMallocHost(&c->host, c->host_bytes) != cudaSuccess) {
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
