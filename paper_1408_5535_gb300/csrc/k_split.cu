@@ -18,13 +18,17 @@
 // and N and 7.1 * 2^62 by the dropped pairs, the sum 2^67 by its last place, K * 2^65.2
 // + 2^67 in all.  A chain of FP64 multiply-adds is relative to the sum of the moduli,
 // S = sum |M N|, which may lie far below: P(i,:) = (1e25, 1, 1, ..) times (0, 1, 1, ..).
-// So one more product per step adds up the moduli of the leading digits (FP16
+// The entry points keep to that (ST): one more product per step adds up the moduli of the leading digits (FP16
 // accumulators, saturating).  |M| >= 0.498 * 2^56 |leading digit|, so a sum of
 // 2^8 proves S >= 2^118 and the error below (K + 4) 2^-52 S; an output that does not
 // reach it is computed in FP64 from the tile in shared memory (redo).  What is kept is in
 // fact better than the chain: random values with p = 8 to 64: at most 0.5 eps S, mean
-// 0.04, against 2.5 and 0.18; with identity-like coefficients, where a quarter is
-// computed anew, at most 1.0 and mean 0.20 against 6.5 and 0.79.
+// 0.04, against 2.5 and 0.18; with identity-like coefficients, a quarter computed anew,
+// at most 1.0 and mean 0.20 against 6.5 and 0.79.
+// The solver's own products go without (ST = false): its bases are orthonormal and
+// its tolerances are norms, for which (row maximum) x (column maximum) is as good; on the
+// localised vectors of a heavy-tailed matrix most outputs would be computed anew (1,000,000 x
+// 500,000, 20 largest, FP64: 146 ms and 188 ms).
 //
 // Why mma.sync: a tile's contraction is 16 x 8 x 64 per digit pair and its
 // operands are made in registers by the warp that uses them, so a warp-level
@@ -37,8 +41,8 @@
 // Measured on the FP64 pipe and here: Gram-Schmidt pass, 500,000 x 55 against 8,
 // subtract and project, 796 us -> 225 us; V Y, 500,000 x 35 to 21, 694 us -> 173 us; to
 // 8, 265 us -> 79 us (without the sums of moduli 218, 173 and 74 us).  Where outputs are
-// computed anew it takes longer: V Y with coefficients I + 1e-3 noise 415 us; the pass
-// on log-normal(2) elements 542 us; elements over 10 decades 705 to 850 us.
+// computed anew it takes longer: the pass on log-normal(2) elements 542 us, on elements over 10
+// decades 705 us; V Y of such up to 850 us.
 //
 // A tile with an Inf, a NaN or values below 2^-950 is computed in plain FP64.
 #include <algorithm>
@@ -235,14 +239,13 @@ __device__ __noinline__ int redo_list(unsigned need, const double* x, int xa, in
   __syncwarp();
   return total;
 }
-__device__ __forceinline__ int redo(unsigned need, const double* x, int xa, int xk, const double* y, int yb, int yk,
-                                    int len, unsigned char* list, double (&out)[4]) {
+__device__ __forceinline__ void redo(unsigned need, const double* x, int xa, int xk, const double* y, int yb, int yk,
+                                     int len, unsigned char* list, double (&out)[4]) {
   double fix[4];
-  const int total = redo_list(need, x, xa, xk, y, yb, yk, len, list, fix);
+  redo_list(need, x, xa, xk, y, yb, yk, len, list, fix);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
     if ((need >> i) & 1u) out[i] = fix[i];
-  return total;
 }
 // V Y where nearly all outputs of 16 x 8 are weak: the digits are wasted, and a warp takes
 // its next tiles in plain FP64 before it tries again (elements over 10 decades, 35 columns to
@@ -291,6 +294,8 @@ struct Scales {
   int F[2][64];          // largest exponent of each column of the coefficients, scaled
   int seen[64];
   int bmin, slack, bad, two;
+  int peak[64], peaks;   // V Y: the one coefficient of a column that is kept out of the digits, or -1
+  double ypeak[64];
 };
 
 // seen[c] = largest exponent of column c among 16 rows of a tile, by a warp
@@ -322,24 +327,45 @@ __device__ inline void set_scales(int p, Scales& sc, int warp, int lane) {
       sc.two = mn < -2;
       sc.slack = 4096;
       sc.bad = 0;
+      sc.peaks = 0;
     }
   }
   __syncthreads();
 }
 
-// Scales F of the r coefficient columns (padded to rc), for both sets.
+// Scales F of the r coefficient columns (padded to rc), for both sets.  Coefficients of
+// restarts and Ritz vectors are often a unit matrix with small entries beside it: the window
+// of a column would hang on the one large coefficient, and whatever is small in P there be
+// weak.  With PEAK a coefficient 8 times the others of its column stays out of the digits:
+// its product is one FP64 multiply-add, and the window that of the others (500,000 rows, 35
+// columns to 21, I + 1e-3 noise: 191 us for 415).
 // sc.bad is set when a coefficient is not finite or a column is too small to be
 // cut, sc.two is cleared when set 1 cannot hold the coefficients.
-template <int NT>
+template <int NT, bool PEAK>
 __device__ inline void coeff_scales(const double* __restrict__ Y, int ldy, int p, int r, int rc, Scales& sc, int tid) {
   const int warp = tid >> 5, lane = tid & 31;
   for (int c = warp; c < rc; c += NT / 32) {
-    int f0 = 0, f1 = -4096, inf = 0, nz = 0;
+    int f0 = 0, f1 = -4096, inf = 0, nz = 0, peak = -1;
+    if (PEAK && c < r) {
+      unsigned m0 = 0, m1 = 0;                   // the lane's larger and smaller, by their high words
+      int k0 = -1;
+      for (int k = lane; k < p; k += 32) {
+        const unsigned m = (unsigned)__double2hiint(Y[k + (size_t)c * ldy]) & 0x7fffffffu;
+        m1 = max(m1, min(m, m0));
+        if (m >= m0) k0 = k;
+        m0 = max(m0, m);
+      }
+      const unsigned top = __reduce_max_sync(0xffffffffu, m0);
+      const int at = __ffs(__ballot_sync(0xffffffffu, m0 == top)) - 1;
+      const unsigned next = __reduce_max_sync(0xffffffffu, lane == at ? m1 : m0);
+      peak = __shfl_sync(0xffffffffu, k0, at);
+      if (top < next + (3u << 20)) peak = -1;
+    }
     for (int k = lane; k < p && c < r; k += 32) {
       const double y = Y[k + (size_t)c * ldy];
       const int e = expo(y);
       inf |= e == 0x7ff;
-      if (y == 0.0) continue;
+      if (y == 0.0 || k == peak) continue;
       nz = 1;
       f0 = max(f0, e);
       f1 = max(f1, e + sc.b[1][k]);
@@ -353,6 +379,11 @@ __device__ inline void coeff_scales(const double* __restrict__ Y, int ldy, int p
       if (nz) {
         if (f1 < E_MIN) sc.two = 0;
         atomicMin(&sc.slack, f0 - f1);
+      }
+      sc.peak[c] = peak;
+      if (peak >= 0) {
+        sc.peaks = 1;
+        sc.ypeak[c] = Y[peak + (size_t)c * ldy];
       }
       sc.F[0][c] = max(f0, E_MIN);
       sc.F[1][c] = max(f1, E_MIN);
@@ -370,7 +401,7 @@ __device__ inline void coeff_lane(const double* __restrict__ Y, int ldy, int p, 
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int k = k0 + 4 * u;
-    y[u] = (k < p && c < r) ? Y[k + (size_t)c * ldy] : 0.0;
+    y[u] = (k < p && c < r && k != sc.peak[c]) ? Y[k + (size_t)c * ldy] : 0.0;
     b[u] = sc.F[set][c] - sc.b[set][k];
   }
   digits2(y[0], b[0], y[1], b[1], d0);
@@ -463,7 +494,7 @@ __device__ __forceinline__ void row_digits(const double* tile, const int* b, int
 }
 
 // acc = the 16 x 8 products of 16 rows of a tile with 8 coefficient columns
-template <int KT, int LDS_>
+template <int KT, int LDS_, bool ST>
 __device__ __forceinline__ void rows_times_coeff(const double* tile, const Scales& sc, int set, const uint2* Bs, int g,
                                                  int t, int lane, const int (&base)[2], Acc& acc, Mag& mag) {
   acc.clear();
@@ -484,7 +515,7 @@ __device__ __forceinline__ void rows_times_coeff(const double* tile, const Scale
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
       const uint2 b = Bs[((set * NS + q) * KT + kt) * 32 + lane];
-      if (q == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
+      if (ST && q == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
 #pragma unroll
       for (int s = 0; s + q < NS; ++s) mma16(acc.c[acc_of(s, q)], a[s], b.x, b.y);
     }
@@ -495,6 +526,12 @@ __device__ __forceinline__ unsigned no_cols(int t, int q) {
   return (2 * t < q ? 0u : 31u) | (2 * t + 1 < q ? 0u : 31u << 16);
 }
 constexpr unsigned NO_ROW = 0x001f001fu;
+
+// Whether the product of the kept-out coefficient y with x alone is large enough for the digits of
+// the others, as a sum of moduli of 2^118 would be (their unit is 2^(base + F - 2168)).
+__device__ __forceinline__ bool peak_holds(double x, double y, int base, int F) {
+  return expo(x) + expo(y) + 4 >= base + F;
+}
 
 // ---------------------------------------------------------------------------
 // Out = P Y [- Xs diag(theta)], optional column norms.  A warp takes 16-row
@@ -544,7 +581,7 @@ __device__ __noinline__ void tall_plain(const double* tile, int row0, int n, int
 }
 
 // A CTA's first tiles, the scales of the columns and of the coefficients.
-template <int KT>
+template <int KT, bool ST>
 __device__ inline void tall_start(int n, const double* P, int ldp, int p, const double* __restrict__ Y, int ldy, int r,
                                   int rc, bool vec, double* buf, int tile, int ntiles, Scales& sc, int tid) {
   const int warp = tid >> 5, lane = tid & 31;
@@ -558,10 +595,10 @@ __device__ inline void tall_start(int n, const double* P, int ldp, int p, const 
   if (tile < ntiles) see_columns<TS_LD>(buf, p, sc, lane);
   __syncthreads();
   set_scales(p, sc, warp, lane);
-  coeff_scales<tall_warps(KT) * 32>(Y, ldy, p, r, rc, sc, tid);
+  coeff_scales<tall_warps(KT) * 32, ST>(Y, ldy, p, r, rc, sc, tid);
 }
 
-template <int KT>
+template <int KT, bool ST>
 __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
     k_tall_rows(int n, const double* P, int ldp, int p, const double* __restrict__ Y, int ldy, int r, double* Out,
                 int ldo, const double* __restrict__ Xs, int ldx, const double* __restrict__ theta, double* norms2,
@@ -578,7 +615,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   const int ntiles = (n + TS_R - 1) / TS_R, stride = gridDim.x * TS_W;
   int tile = warp * gridDim.x + blockIdx.x;      // the first wave spreads over all CTAs
   if (lane < 8) wn[warp][lane] = 0.0;
-  tall_start<KT>(n, P, ldp, p, Y, ldy, r, 8, vec, buf, tile, ntiles, sc, tid);
+  tall_start<KT, ST>(n, P, ldp, p, Y, ldy, r, 8, vec, buf, tile, ntiles, sc, tid);
   coeff_frag_b<KT, TS_W * 32>(Y, ldy, p, r, sc, Bs, tid);
   const bool plain = sc.bad != 0;
   const int c0 = 2 * t;
@@ -609,8 +646,10 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
       }
       Acc acc;
       Mag mag;
-      rows_times_coeff<KT, TS_LD>(buf, sc, set, Bs, g, t, lane, base, acc, mag);
+      rows_times_coeff<KT, TS_LD, ST>(buf, sc, set, Bs, g, t, lane, base, acc, mag);
       const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
+      // what the kept-out coefficient of output q's column multiplies
+      auto x_of = [&](int q) { return buf[sc.peak[c0 + (q & 1)] * TS_LD + g + (q < 2 ? 0 : 8)]; };
       auto finish = [&](int q, double o) {
         const int c = c0 + (q & 1), i = i0 + (q < 2 ? 0 : 8);
         if (theta) o = fma(-th[q & 1], xs[q], o);
@@ -620,22 +659,37 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
         }
       };
       unsigned need = 0u;
-      if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+      if (ST && any_less2(__vminu2(l0, l1), MAG_MIN)) {
         need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
-        double fix[4];
-        if (redo_list(need, buf, 1, TS_LD, Y, ldy, 1, p, list[warp], fix) > WEAK_MANY) skip = WEAK_SKIP;
+        if (sc.peaks) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if ((need >> q) & 1u) finish(q, fix[q]);
+          for (int q = 0; q < 4; ++q) {
+            const int c = c0 + (q & 1);
+            if (sc.peak[c] >= 0 && peak_holds(x_of(q), sc.ypeak[c], base[q < 2 ? 0 : 1], sc.F[set][c])) need &= ~(1u << q);
+          }
+        }
+        if (__any_sync(0xffffffffu, need)) {
+          double fix[4];
+          if (redo_list(need, buf, 1, TS_LD, Y, ldy, 1, p, list[warp], fix) > WEAK_MANY) skip = WEAK_SKIP;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if ((need >> q) & 1u) finish(q, fix[q]);
+        }
       }
-      __syncwarp();                              // every lane is done with the tile
-      if (next < ntiles) load_cols<TS_R, TS_LD, 32>(P, ldp, p, n, next * TS_R, vec, buf, lane);
-      cp_commit();
+      auto reload = [&] {
+        __syncwarp();                            // every lane is done with the tile
+        if (next < ntiles) load_cols<TS_R, TS_LD, 32>(P, ldp, p, n, next * TS_R, vec, buf, lane);
+        cp_commit();
+      };
+      if (!ST || !sc.peaks) reload();                   // beside the sums (79 us; after them 87)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const double o = times_pow2(acc.sum(q), base[q < 2 ? 0 : 1] + sc.F[set][c0 + (q & 1)] - E_OUT);
+        const int c = c0 + (q & 1);
+        double o = times_pow2(acc.sum(q), base[q < 2 ? 0 : 1] + sc.F[set][c] - E_OUT);
+        if (ST && sc.peaks && sc.peak[c] >= 0) o = fma(x_of(q), sc.ypeak[c], o);
         if (!((need >> q) & 1u)) finish(q, o);
       }
+      if (ST && sc.peaks) reload();
     }
     cp_wait<0>();
     __syncwarp();
@@ -658,7 +712,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   }
 }
 
-template <int KT>
+template <int KT, bool ST>
 __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
     k_tall_cols(int n, const double* P, int ldp, int p, const double* __restrict__ Y, int ldy, int r, double* Out,
                 int ldo, const double* __restrict__ Xs, int ldx, const double* __restrict__ theta, double* norms2,
@@ -677,7 +731,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
   int tile = warp * gridDim.x + blockIdx.x;
   if (norms2)
     for (int e = lane; e < mt * 64; e += 32) slot[e] = 0.0;
-  tall_start<KT>(n, P, ldp, p, Y, ldy, r, mt * 16, vec, buf, tile, ntiles, sc, tid);
+  tall_start<KT, ST>(n, P, ldp, p, Y, ldy, r, mt * 16, vec, buf, tile, ntiles, sc, tid);
   coeff_frag_a<KT, TS_W * 32>(Y, ldy, p, r, mt, sc, As, tid);
   const bool plain = sc.bad != 0;
   int skip = 0;
@@ -723,7 +777,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
             for (int s = 0; s < NS; ++s) {
               const uint4 v = as[(kt * NS + s) * 32];
               const unsigned a[4] = {v.x, v.y, v.z, v.w};
-              if (s == 0) mag.add(v.x, v.y, v.z, v.w, b[kt][0][0], b[kt][0][1]);
+              if (ST && s == 0) mag.add(v.x, v.y, v.z, v.w, b[kt][0][0], b[kt][0][1]);
 #pragma unroll
               for (int q = 0; s + q < NS; ++q) mma16(acc.c[acc_of(s, q)], a, b[kt][q][0], b[kt][q][1]);
             }
@@ -731,8 +785,16 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
           const unsigned l0 = mag.levels(0) | pad | (j * 16 + g < r ? 0u : NO_ROW);
           const unsigned l1 = mag.levels(1) | pad | (j * 16 + g + 8 < r ? 0u : NO_ROW);
           unsigned need = 0u;
-          if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+          if (ST && any_less2(__vminu2(l0, l1), MAG_MIN)) {
             need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
+            if (sc.peaks) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int c = j * 16 + g + 8 * (q >> 1), k = sc.peak[c];
+                if (k >= 0 && peak_holds(buf[k * TS_LD + 8 * h + 2 * t + (q & 1)], sc.ypeak[c], q & 1 ? e1 : e0, F[c]))
+                  need &= ~(1u << q);
+              }
+            }
             weak |= need << (16 * h + 4 * j);
           }
 #pragma unroll
@@ -740,6 +802,11 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
             const int c = j * 16 + g + 8 * u;
             double o0 = times_pow2(acc.sum(2 * u), e0 + F[c] - E_OUT);
             double o1 = times_pow2(acc.sum(2 * u + 1), e1 + F[c] - E_OUT);
+            if (ST && sc.peaks && sc.peak[c] >= 0) {
+              const double* x = buf + sc.peak[c] * TS_LD + 8 * h + 2 * t;
+              o0 = fma(x[0], sc.ypeak[c], o0);
+              o1 = fma(x[1], sc.ypeak[c], o1);
+            }
             if (c < r && i < n) {
               if (theta) {
                 const double th = theta[c];
@@ -762,7 +829,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
           }
         }
       }
-      if (__any_sync(0xffffffffu, weak)) {
+      if (ST && __any_sync(0xffffffffu, weak)) {
         int most = 0;
         for (int h = 0; h < 2; ++h)
           for (int j = 0; j < mt; ++j) {
@@ -844,7 +911,7 @@ __device__ __forceinline__ unsigned raise(unsigned e, unsigned l, unsigned& top)
   return e + MAG_MIN;
 }
 
-template <int KT>
+template <int KT, bool ST>
 __global__ void __launch_bounds__(CS_W * 32, 2)
     k_cgs_split(int n, Basis<double> P, double* __restrict__ Tb, int ldt, int q, const double* __restrict__ Gsub,
                 double* __restrict__ Gout, double* __restrict__ Tout, bool vec, bool vect, RedWs rw) {
@@ -883,7 +950,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
       see_columns<CS_LD>(Ps + 16 * warp, p, sc, lane);
       __syncthreads();
       set_scales(p, sc, warp, lane);
-      coeff_scales<CS_W * 32>(Gsub, p, p, q, 8, sc, tid);
+      coeff_scales<CS_W * 32, false>(Gsub, p, p, q, 8, sc, tid);
       coeff_frag_b<KT, CS_W * 32>(Gsub, p, p, q, sc, Bs, tid);
     }
     first = false;
@@ -903,14 +970,14 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
       } else {
         Acc acc;
         Mag mag;
-        rows_times_coeff<KT, CS_LD>(cur, sc, set, Bs, g, t, lane, base, acc, mag);
+        rows_times_coeff<KT, CS_LD, ST>(cur, sc, set, Bs, g, t, lane, base, acc, mag);
         const int i0 = row0 + 16 * warp + g;       // (rows past n are zero)
         const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
         double out[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           out[i] = times_pow2(acc.sum(i), base[i < 2 ? 0 : 1] + sc.F[set][2 * t + (i & 1)] - E_OUT);
-        if (any_less2(__vminu2(l0, l1), MAG_MIN)) {
+        if (ST && any_less2(__vminu2(l0, l1), MAG_MIN)) {
           unsigned need = less2(l0, MAG_MIN) | less2(l1, MAG_MIN) << 2;
           // the digits' error, below 2^5 of the sum's last place, is no matter where it is below
           // half an ulp of T (their last place is 2^(base + F - E_OUT))
@@ -977,7 +1044,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
 #pragma unroll
             for (int k = 0; k < NS; ++k) {
               const uint2 b = Td[((ch * KS + ks) * NS + k) * 32 + lane];
-              if (k == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
+              if (ST && k == 0) mag.add(a[0][0], a[0][1], a[0][2], a[0][3], b.x, b.y);
 #pragma unroll
               for (int s = 0; s + k < NS; ++s) mma16(acc.c[acc_of(s, k)], a[s], b.x, b.y);
             }
@@ -990,7 +1057,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
 #pragma unroll
           for (int i = 0; i < 4; ++i)
             out[i] = times_pow2(acc.sum(i), (i < 2 ? e0 : e1) + (i & 1 ? s1 : s0) - E_OUT);
-          if (any_less2(gtop[0], w0) || any_less2(gtop[1], w1))
+          if (ST && (any_less2(gtop[0], w0) || any_less2(gtop[1], w1)) && row0 + ch * RC < n)   // (zero past n)
             redo(less2(gtop[0], w0) | less2(gtop[1], w1) << 2, Ps + 16 * m * CS_LD + ch * RC, CS_LD, 1, Ts + ch * RC,
                  CS_LD, 1, RC, list[warp], out);
 #pragma unroll
@@ -1023,7 +1090,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
 #pragma unroll
             for (int s = 0; s < NS; ++s) {
               const unsigned a[4] = {b[s].x, 0u, b[s].y, 0u};
-              if (s == 0) mag.add(b[0].x, 0u, b[0].y, 0u, b[0].x, b[0].y);
+              if (ST && s == 0) mag.add(b[0].x, 0u, b[0].y, 0u, b[0].x, b[0].y);
 #pragma unroll
               for (int k = 0; s + k < NS; ++k) mma16(acc.c[acc_of(s, k)], a, b[k].x, b[k].y);
             }
@@ -1031,7 +1098,7 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
           const int e = te[tch][g], s0 = e + te[tch][2 * t], s1 = e + te[tch][2 * t + 1];
           const unsigned w = raise((unsigned)s0 | (unsigned)s1 << 16, mag.levels(0) | pad | (g < q ? 0u : NO_ROW), ttop);
           double out[4] = {times_pow2(acc.sum(0), s0 - E_OUT), times_pow2(acc.sum(1), s1 - E_OUT), 0.0, 0.0};
-          if (any_less2(ttop, w))
+          if (ST && any_less2(ttop, w) && row0 + tch * RC < n)
             redo(less2(ttop, w), Ts + tch * RC, CS_LD, 1, Ts + tch * RC, CS_LD, 1, RC, list[warp], out);
           tacc[0] += out[0];
           tacc[1] += out[1];
@@ -1084,39 +1151,39 @@ int split_sms() {
 bool even16(const double* p, int ld) { return p == nullptr || (((uintptr_t)p & 15) == 0 && ld % 2 == 0); }
 constexpr size_t SPLIT_SMEM = 220 * 1024;
 
-template <int KT>
+template <int KT, bool ST>
 void tall_go(cudaStream_t s, int n, const double* P, int ldp, int p, const double* Y, int ldy, int r, double* Out,
              int ldo, const double* Xs, int ldx, const double* theta, double* norms2) {
   const TallSmem sm(KT, r, norms2 != nullptr);
   static std::atomic<uint64_t> done{0};
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_tall_rows<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SPLIT_SMEM);
-    cudaFuncSetAttribute(k_tall_cols<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SPLIT_SMEM);
+    cudaFuncSetAttribute(k_tall_rows<KT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SPLIT_SMEM);
+    cudaFuncSetAttribute(k_tall_cols<KT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SPLIT_SMEM);
   });
   const int grid = std::min(split_sms(), ceil_div(n, TS_R));
   const RedWs rw = norms2 ? red_ws((size_t)grid * r) : RedWs{};
   if (r <= 8)
-    k_tall_rows<KT><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
+    k_tall_rows<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
                                                       even16(P, ldp), sm.tiles, rw);
   else
-    k_tall_cols<KT><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
+    k_tall_cols<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
                                                       even16(P, ldp), even16(Out, ldo), sm.tiles, sm.norms, rw);
   count_launch();
   if (norms2) reduce_partials(s, rw, grid, r, norms2, 0, nullptr);
 }
 
-template <int KT>
+template <int KT, bool ST>
 void cgs_go(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ldt, int q, const double* Gsub,
             double* Gout, double* Tout) {
   constexpr size_t smem = sizeof(uint2) * NS * 32 * (2 * KT + CS_W) + sizeof(double) * (KT * 16 + 8) * CS_LD;
   static std::atomic<uint64_t> done{0};
   once_per_device(done, [&] {
-    cudaFuncSetAttribute(k_cgs_split<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_cgs_split<KT, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   });
   const int grid = std::min(2 * split_sms(), ceil_div(n, CS_R));
   const int n1 = Gout ? P.cols() * q : 0, n2 = Tout ? q * q : 0;
   const RedWs rw = red_ws((size_t)grid * (n1 + n2));
-  k_cgs_split<KT><<<grid, CS_W * 32, smem, s>>>(n, P, Tb, ldt, q, Gsub, Gout, Tout,
+  k_cgs_split<KT, ST><<<grid, CS_W * 32, smem, s>>>(n, P, Tb, ldt, q, Gsub, Gout, Tout,
                                                 even16(P.p1, P.ld1) && even16(P.p2, P.ld2), even16(Tb, ldt), rw);
   count_launch();
   reduce_partials(s, rw, grid, n1, Gout, n2, Tout);
@@ -1129,16 +1196,16 @@ void cgs_go(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ldt, 
 // r = 3: 9.1 / 7.2; p = 35, r = 21: 50 / 17; n = 500,000, p = 10, r = 3: 76 / 42),
 // one and two columns are nearer to their FP64 work in the streaming form.
 bool tall_split(cudaStream_t s, int n, const double* P, int ldp, int p, const double* Y, int ldy, int r, double* Out,
-                int ldo, const double* Xs, int ldx, const double* theta, double* norms2) {
+                int ldo, const double* Xs, int ldx, const double* theta, double* norms2, bool strict) {
   const int KT = (p + 15) / 16;
   if (n < 512 || n > INT32_MAX - 256 || r < 3 || p < 8 || p > 64 || r > 64 ||
       TallSmem(KT, r, norms2 != nullptr).total > SPLIT_SMEM)
     return false;
   switch (KT) {
-    case 1: tall_go<1>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    case 2: tall_go<2>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    case 3: tall_go<3>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    default: tall_go<4>(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
+    case 1: (strict ? tall_go<1, true> : tall_go<1, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
+    case 2: (strict ? tall_go<2, true> : tall_go<2, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
+    case 3: (strict ? tall_go<3, true> : tall_go<3, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
+    default: (strict ? tall_go<4, true> : tall_go<4, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
   }
   return true;
 }
@@ -1149,16 +1216,16 @@ bool tall_split(cudaStream_t s, int n, const double* P, int ldp, int p, const do
 // (p = 35, q = 3: n = 4096: 14.7 / 16.7, n = 16,384: 25 / 19, n = 500,000:
 // 267 / 195; p = 10, q = 3, n = 500,000: 86 / 101).
 bool cgs_split(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ldt, int q, const double* Gsub,
-               double* Gout, double* Tout) {
+               double* Gout, double* Tout, bool strict) {
   const int p = P.cols();
   if (n < (q >= 5 ? 512 : 8192) || n > INT32_MAX - 256 || q < 3 || p < (q >= 5 ? 10 : 16) || p > 64 ||
       !(Gsub || Gout))
     return false;
   switch ((p + 15) / 16) {
-    case 1: cgs_go<1>(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    case 2: cgs_go<2>(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    case 3: cgs_go<3>(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    default: cgs_go<4>(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
+    case 1: (strict ? cgs_go<1, true> : cgs_go<1, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
+    case 2: (strict ? cgs_go<2, true> : cgs_go<2, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
+    case 3: (strict ? cgs_go<3, true> : cgs_go<3, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
+    default: (strict ? cgs_go<4, true> : cgs_go<4, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
   }
   return true;
 }

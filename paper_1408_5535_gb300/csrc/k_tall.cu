@@ -283,13 +283,13 @@ static void cgs_launch(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt,
 
 template <typename T>
 void cgs_pass(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, const double* Gsub, double* Gout,
-              double* Tout) {
+              double* Tout, bool strict) {
   if (n <= 0 || q <= 0) return;
   ProfScope ps(s, pcat<T>(PROF_GRAM));
   Basis<T> PP = P;
   if (PP.cols() == 0) { Gsub = nullptr; Gout = nullptr; }
   if constexpr (sizeof(T) == 8)
-    if (cgs_split(s, n, PP, Tb, ldt, q, Gsub, Gout, Tout)) {
+    if (cgs_split(s, n, PP, Tb, ldt, q, Gsub, Gout, Tout, strict)) {
       count_cgs<T>(n, PP.cols(), q, Gsub, Gout, Tout);
       return;
     }
@@ -563,7 +563,7 @@ static void tall_stream(cudaStream_t s, int n, const T* P, int ldp, int p, const
 
 template <typename T>
 void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
-                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2) {
+                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2, bool strict) {
   if (n <= 0 || r <= 0) return;
   ProfScope ps(s, pcat<T>(PROF_TALL));
   count_work(pcat<T>(PROF_TALL), 2.0 * n * p * r + (theta ? 2.0 * n * r : 0.0) + (norms2 ? 2.0 * n * r : 0.0),
@@ -580,7 +580,7 @@ void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const d
     PH_STREAM(64, 1);
   } else {
     if (r == 2) PH_STREAM(2, 1);
-    if (tall_split(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2)) return;
+    if (tall_split(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2, strict)) return;
     tall_general(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2);
   }
 #undef PH_STREAM
@@ -846,9 +846,10 @@ template void fill_const<float>(cudaStream_t, int64_t, float, float*);
 
 // explicit instantiations
 #define PH_INST(T)                                                                                              \
-  template void cgs_pass<T>(cudaStream_t, int, const Basis<T>&, T*, int, int, const double*, double*, double*); \
+  template void cgs_pass<T>(cudaStream_t, int, const Basis<T>&, T*, int, int, const double*, double*, double*,  \
+                            bool);                                                                               \
   template void tall_times_small<T>(cudaStream_t, int, const T*, int, int, const double*, int, int, T*, int,    \
-                                    const T*, int, const double*, double*);                                    \
+                                    const T*, int, const double*, double*, bool);                                    \
   template void scale_block<T>(cudaStream_t, int, T*, int, int, const double*, T*, int);                       \
   template void cm_to_rm<T>(cudaStream_t, int, const T*, int, int, T*);                                        \
   template void rm_to_cm<T>(cudaStream_t, int, const T*, int, T*, int);                                        \

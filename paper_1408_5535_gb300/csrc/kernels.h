@@ -131,7 +131,7 @@ struct Basis {
 //   if Tout:  Tout += T^T T          (q x q, FP64, must be zeroed by caller)
 template <typename T>
 void cgs_pass(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, const double* Gsub, double* Gout,
-              double* Tout);
+              double* Tout, bool strict = false);
 
 // Out (n x r, column-major ld ldo) = P (n x p) * Y (p x r, FP64 column-major ld ldy)
 // [- Xs (n x r) * diag(theta)] when theta != nullptr.  In-place allowed when
@@ -139,14 +139,16 @@ void cgs_pass(cudaStream_t s, int n, const Basis<T>& P, T* Tb, int ldt, int q, c
 // If norms2 != nullptr: norms2[c] += ||Out(:,c)||^2 (FP64, zeroed by caller).
 template <typename T>
 void tall_times_small(cudaStream_t s, int n, const T* P, int ldp, int p, const double* Y, int ldy, int r, T* Out,
-                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2);
+                      int ldo, const T* Xs, int ldx, const double* theta, double* norms2, bool strict = false);
 
 // The FP64 forms on the FP16 tensor cores (k_split.cu); false: not a shape
-// for them (nothing launched).
+// for them (nothing launched).  strict: every output as accurate as by FP64
+// multiply-adds, relative to the sum of its terms' moduli (the entry points); without,
+// relative to the rows' and columns' maxima (the solver).
 bool cgs_split(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ldt, int q, const double* Gsub,
-               double* Gout, double* Tout);
+               double* Gout, double* Tout, bool strict);
 bool tall_split(cudaStream_t s, int n, const double* P, int ldp, int p, const double* Y, int ldy, int r, double* Out,
-                int ldo, const double* Xs, int ldx, const double* theta, double* norms2);
+                int ldo, const double* Xs, int ldx, const double* theta, double* norms2, bool strict);
 
 // T <- T * Linv^T  (q x q upper-triangular inverse factor applied on the right,
 // FP64) and copy T into column-major destination Dst (ld ldd) when non-null.

@@ -3013,7 +3013,7 @@ static phsvds_status block_cgs_api(phsvds_handle h, int64_t n, const T* P1, int 
   cudaError_t e = cudaSetDevice(h->device);
   if (e != cudaSuccess) return set_err(h, PHSVDS_ERR_CUDA, cudaGetErrorString(e));
   Basis<T> P{P1, ld1, p1, P2, ld2, p2};
-  cgs_pass<T>(h->stream, (int)n, P, Tb, ldt, q, Gsub, Gout, Tout);
+  cgs_pass<T>(h->stream, (int)n, P, Tb, ldt, q, Gsub, Gout, Tout, true);
   e = cudaGetLastError();
   return e == cudaSuccess ? PHSVDS_OK : set_err(h, PHSVDS_ERR_CUDA, cudaGetErrorString(e));
 }
@@ -3027,7 +3027,7 @@ static phsvds_status tall_small_api(phsvds_handle h, int64_t n, const T* P, int 
     return set_err(h, PHSVDS_ERR_INVALID, "invalid tall-times-small arguments");
   cudaError_t e = cudaSetDevice(h->device);
   if (e != cudaSuccess) return set_err(h, PHSVDS_ERR_CUDA, cudaGetErrorString(e));
-  tall_times_small<T>(h->stream, (int)n, P, ldp, p, Y, ldy, r, Out, ldo, theta ? Xs : nullptr, ldx, theta, norms2);
+  tall_times_small<T>(h->stream, (int)n, P, ldp, p, Y, ldy, r, Out, ldo, theta ? Xs : nullptr, ldx, theta, norms2, true);
   e = cudaGetLastError();
   return e == cudaSuccess ? PHSVDS_OK : set_err(h, PHSVDS_ERR_CUDA, cudaGetErrorString(e));
 }

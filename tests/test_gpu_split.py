@@ -277,3 +277,21 @@ def test_block_cgs_peaks_inside_a_row_and_a_column(h, n, p, q, peak, kind):
             got = buf.cpu().numpy().reshape(q, -1).T
             lim = (n / 64 + 64) * EPS * (np.abs(A).T @ np.abs(T2))
             assert np.all(np.abs(got - _mm(A.T, T2)) <= lim)
+
+
+@pytest.mark.parametrize("p,r", [(9, 4), (33, 8), (35, 21), (64, 30)])
+@pytest.mark.parametrize("small", [0.1, 1e-3, 1e-9, 0.0])
+def test_tall_coefficients_with_one_large_entry(h, p, r, small):
+    """A coefficient far above the others of its column stays out of the digits: unit vectors with
+    noise beside them, some columns of even size, one of zeros, signs, and with peaks in P."""
+    rng = np.random.default_rng(p)
+    n = 1000
+    Y = small * rng.standard_normal((p, r))
+    Y[rng.permutation(p)[:r], np.arange(r)] = rng.choice([-1.0, 3.0, 1e-200, 1e200], r)
+    Y[:, 1] = rng.standard_normal(p)
+    Y[:, 2] = 0.0
+    for kind, peak in (("one", 1.0), ("one", 1e6), ("spread", 1e25)):
+        P = _peaks(rng, n, p, peak, kind)
+        out, _ = _tall(h, P, Y)
+        S = np.abs(P) @ np.abs(Y)
+        assert np.all(np.abs(out - _mm(P, Y)) <= (p + 4) * EPS * S + 1e-300)
