@@ -440,11 +440,13 @@ __global__ void __launch_bounds__(CSC_TH) k_scatter_csc(int m, const int* __rest
 // holds up to SORT_R words and counts the words below each of them.  Longer
 // columns are left to the whole CTA, one after another: a sorting network of
 // compare-exchanges towards the lower index (which sorts any length, as if it
-// were padded at the end with the largest key), in place.
+// were padded at the end with the largest key), in place.  Entries past row_ptr[m]
+// are counted but have no row and so no word: what their slots hold is not an index.
 constexpr int SORT_R = 4;
 template <int L>
-__global__ void __launch_bounds__(CSC_TH) k_sort_cols(int n, const int* __restrict__ cp, const double* __restrict__ va,
-                                                      int* __restrict__ ri, double* __restrict__ cv) {
+__global__ void __launch_bounds__(CSC_TH) k_sort_cols(int n, int64_t nnz, const int* __restrict__ cp,
+                                                      const double* __restrict__ va, int* __restrict__ ri,
+                                                      double* __restrict__ cv) {
   __shared__ int long_cols[CSC_TH / L];
   __shared__ int nlong;
   if (threadIdx.x == 0) nlong = 0;
@@ -480,7 +482,7 @@ __global__ void __launch_bounds__(CSC_TH) k_sort_cols(int n, const int* __restri
   double v[SORT_R];
 #pragma unroll
   for (int u = 0; u < SORT_R; ++u)
-    if (mine && u * L + lane < len) v[u] = va[w[u] >> 32];
+    if (mine && u * L + lane < len) v[u] = (int64_t)(w[u] >> 32) < nnz ? va[w[u] >> 32] : 0.0;
   __syncwarp();
 #pragma unroll
   for (int u = 0; u < SORT_R; ++u)
@@ -514,7 +516,7 @@ __global__ void __launch_bounds__(CSC_TH) k_sort_cols(int n, const int* __restri
     for (int64_t k = threadIdx.x; k < ln; k += CSC_TH) {
       const unsigned long long x = a[k];
       ri[s0 + k] = (int)(unsigned)x;
-      cv[s0 + k] = va[x >> 32];
+      cv[s0 + k] = (int64_t)(x >> 32) < nnz ? va[x >> 32] : 0.0;
     }
     __syncthreads();
   }
@@ -552,11 +554,11 @@ void csr_to_csc(cudaStream_t s, int m, int n, int64_t nnz, const int* rp, const 
   // slots whatever the column's length, so L * SORT_R is kept near its mean
   // length (with room for its spread)
   if (col <= 6.0)
-    k_sort_cols<4><<<ceil_div((int64_t)n * 4, CSC_TH), CSC_TH, 0, s>>>(n, cp, va, ri, cv);
+    k_sort_cols<4><<<ceil_div((int64_t)n * 4, CSC_TH), CSC_TH, 0, s>>>(n, nnz, cp, va, ri, cv);
   else if (col <= 16.0)
-    k_sort_cols<8><<<ceil_div((int64_t)n * 8, CSC_TH), CSC_TH, 0, s>>>(n, cp, va, ri, cv);
+    k_sort_cols<8><<<ceil_div((int64_t)n * 8, CSC_TH), CSC_TH, 0, s>>>(n, nnz, cp, va, ri, cv);
   else if (col <= 40.0)
-    k_sort_cols<16><<<ceil_div((int64_t)n * 16, CSC_TH), CSC_TH, 0, s>>>(n, cp, va, ri, cv);
+    k_sort_cols<16><<<ceil_div((int64_t)n * 16, CSC_TH), CSC_TH, 0, s>>>(n, nnz, cp, va, ri, cv);
   else
     k_sort_cols<32><<<ceil_div((int64_t)n * 32, CSC_TH), CSC_TH, 0, s>>>(n, cp, va, ri, cv);
   count_launch();

@@ -40,3 +40,29 @@ def test_csr_to_csc_column_lengths(h, m, n, row, dense):
     assert np.array_equal(cp.cpu().numpy(), T.indptr)
     assert np.array_equal(ri.cpu().numpy()[: S.nnz], T.indices)
     assert np.array_equal(cv.cpu().numpy()[: S.nnz], T.data)
+
+
+@pytest.mark.parametrize("n,stray", [(300, 7), (40, 5000)])
+def test_entries_past_the_last_row_are_not_followed(h, n, stray):
+    """nnz larger than row_ptr[m] (a buffer with room to spare): the entries past the last
+    row have no row, all in column 0 here; the other columns are as they should be, and what
+    was in the output buffers is not taken for an index."""
+    m = 500
+    rng = np.random.default_rng(n)
+    S = sp.random(m, n, density=0.05, format="csr", random_state=rng, data_rvs=rng.standard_normal)
+    S.sort_indices()
+    T = S.tocsc()
+    T.sort_indices()
+    dev = lambda a, t: torch.from_numpy(np.ascontiguousarray(a.astype(t))).cuda()
+    nnz = S.nnz + stray
+    cp = torch.full((n + 1,), -1, dtype=torch.int32, device="cuda")
+    ri = torch.full((nnz,), -1, dtype=torch.int32, device="cuda")
+    cv = torch.full((nnz,), 1e300, dtype=torch.float64, device="cuda")
+    ci = np.concatenate([S.indices, np.zeros(stray, S.indices.dtype)])
+    va = np.concatenate([S.data, np.ones(stray)])
+    native.phsvds_csr_to_csc(h, m, n, nnz, dev(S.indptr, np.int32), dev(ci, np.int32), dev(va, np.float64), cp, ri, cv)
+    native.phsvds_sync(h)
+    a = T.indptr[1]
+    assert np.array_equal(cp.cpu().numpy()[1:], T.indptr[1:] + stray)
+    assert np.array_equal(ri.cpu().numpy()[a + stray:], T.indices[a:])
+    assert np.array_equal(cv.cpu().numpy()[a + stray:], T.data[a:])
