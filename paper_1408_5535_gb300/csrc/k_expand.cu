@@ -11,7 +11,10 @@
 // distributed shared memory in a fixed order, and every CTA factorises alike.
 //   warps x 4 columns    G = P^T T: lanes over the rows, butterflies in T, CTAs in FP64
 //   rows x LG lanes      T -= P G: LG lanes share the columns of a row
-// Precision is the general form's: partial sums in T over a few rows, FP64 across CTAs.
+// Sums are as accurate as the general form's, which adds two terms per lane and a warp's
+// lanes in T, and FP64 from there.  A lane has up to 63 terms here: in FP32 it adds four at
+// a time, and these, as the lanes, with the rounding error carried along (two_sum), FP64
+// across CTAs; in FP64 plainly.
 //
 // Time per iteration of stage 1 with the general form and with this one (2n x n, 8 entries
 // per row, 35 basis vectors at most, blocks of 1, 4, 8):
@@ -96,6 +99,39 @@ __device__ bool warp_chol(int q, const double* P, const double* ref, double drop
   return bad;
 }
 
+// hi + lo = the sum so far plus v, to twice FP32 (Knuth's TwoSum: exact for hi + v).
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
+  const float s = __fadd_rn(hi, v), z = __fadd_rn(s, -hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -z)), __fadd_rn(v, -z)));
+  hi = s;
+}
+// As reduce_scatter, of sums hi + lo.
+template <int N, int O, int CUR>
+__device__ __forceinline__ void reduce_scatter2(float (&hi)[N], float (&lo)[N], int lane) {
+  if constexpr (O > 0) {
+    constexpr int H = CUR > 1 ? CUR / 2 : 1;
+    const bool up = CUR > 1 && (lane & O) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      float a = hi[i], b = lo[i], sa = a, sb = b;  // what the lane keeps and what it sends
+      if constexpr (CUR > 1) {
+        if (up) {
+          a = hi[i + H];
+          b = lo[i + H];
+        } else {
+          sa = hi[i + H];
+          sb = lo[i + H];
+        }
+      }
+      const float ra = __shfl_xor_sync(0xffffffffu, sa, O), rb = __shfl_xor_sync(0xffffffffu, sb, O);
+      two_sum(a, b, ra);
+      hi[i] = a;
+      lo[i] = __fadd_rn(b, rb);
+    }
+    reduce_scatter2<N, O / 2, H>(hi, lo, lane);
+  }
+}
+
 template <typename T, int Q>
 __global__ void __launch_bounds__(XT, 1) k_expand_cluster(ExArgs g) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -125,34 +161,64 @@ __global__ void __launch_bounds__(XT, 1) k_expand_cluster(ExArgs g) {
     __syncthreads();
     for (int l0 = warp * XC; l0 < L; l0 += XW * XC) {
       const T* pc[XC];
-      T s[XC * Q];
 #pragma unroll
       for (int a = 0; a < XC; ++a) {
         const int l = l0 + a;
         pc[a] = l < c1 ? Xl + (size_t)l * n : l < c1 + c2 ? V + (size_t)(l - c1) * n : l < L ? ts + (l - c1 - c2) * R
                                                                                             : ts;
       }
+      T s[XC * Q];
 #pragma unroll
       for (int k = 0; k < XC * Q; ++k) s[k] = T(0);
-#pragma unroll 2
-      for (int i = lane; i < nr; i += 32) {
-        T x[XC];
+      double total;
+      if constexpr (sizeof(T) == 4) {
+        constexpr int U = 4;                       // rows whose products are added plainly
+        T lo[XC * Q];
 #pragma unroll
-        for (int a = 0; a < XC; ++a) x[a] = pc[a][i];
+        for (int k = 0; k < XC * Q; ++k) lo[k] = T(0);
+        for (int i = lane; i < nr; i += 32 * U) {
+          T x[U][XC];
 #pragma unroll
-        for (int r = 0; r < Q; ++r) {
-          const T t = ts[r * R + i];
+          for (int u = 0; u < U; ++u)
 #pragma unroll
-          for (int a = 0; a < XC; ++a) s[a * Q + r] = fma(x[a], t, s[a * Q + r]);
+            for (int a = 0; a < XC; ++a) x[u][a] = i + 32 * u < nr ? pc[a][i + 32 * u] : T(0);
+#pragma unroll
+          for (int r = 0; r < Q; ++r) {
+            T t[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) t[u] = i + 32 * u < nr ? ts[r * R + i + 32 * u] : T(0);
+#pragma unroll
+            for (int a = 0; a < XC; ++a) {
+              T v = x[0][a] * t[0];
+#pragma unroll
+              for (int u = 1; u < U; ++u) v = fma(x[u][a], t[u], v);
+              two_sum(s[a * Q + r], lo[a * Q + r], v);
+            }
+          }
         }
+        reduce_scatter2<XC * Q, 16, XC * Q>(s, lo, lane);
+        total = (double)s[0] + (double)lo[0];
+      } else {
+#pragma unroll 2
+        for (int i = lane; i < nr; i += 32) {
+          T x[XC];
+#pragma unroll
+          for (int a = 0; a < XC; ++a) x[a] = pc[a][i];
+#pragma unroll
+          for (int r = 0; r < Q; ++r) {
+            const T t = ts[r * R + i];
+#pragma unroll
+            for (int a = 0; a < XC; ++a) s[a * Q + r] = fma(x[a], t, s[a * Q + r]);
+          }
+        }
+        reduce_scatter<T, XC * Q>(s, lane);
+        total = s[0];
       }
-      reduce_scatter<T, XC * Q>(s, lane);
       constexpr int REP = 32 / (XC * Q);           // lanes that hold the same sum
       const int o = l0 * Q + lane / REP;
-      if (o < L * Q) {
-        const double v = (double)s[0];
-        for (int r = lane % REP; r < nc; r += REP) *cl.map_shared_rank(slot + ((size_t)par * nc + cr) * g.cap + o, r) = v;
-      }
+      if (o < L * Q)
+        for (int r = lane % REP; r < nc; r += REP)
+          *cl.map_shared_rank(slot + ((size_t)par * nc + cr) * g.cap + o, r) = total;
     }
     cl.sync();
     for (int o = tid; o < L * Q; o += XT) {
