@@ -35,33 +35,97 @@ __device__ __forceinline__ void ld_row(const T* p, T (&r)[Q]) {
 }
 
 // out(row, :) = sum of val * X(col, :) over the entries of rows [r0, r1), L lanes
-// per row, JT threads; row(i, acc) is called by the first lane of the group.
+// per row, JT threads; row(i, acc) is called by one thread.  A row much longer than the
+// mean would keep its lanes, and the cluster behind them, for len / L dependent gathers (one
+// full row of 12,000 beside 6 entries per row: 2583 us per iteration of stage 1 for 185).
+// Rows over ROW_LANE L entries wait for a whole warp, over ROW_WARP for the CTA: a rule of
+// the length alone, so that sums repeat.
+constexpr int ROW_LANE = 64, ROW_WARP = 4096;
+constexpr int ROW_BIG = 512;   // more rows of ROW_WARP entries than the lines of the kernels let in
+template <typename T, int Q>
+__device__ __forceinline__ void spmm_add(const int* __restrict__ idx, const T* __restrict__ val, const T* X, int e,
+                                         int e1, int step, T (&acc)[Q]) {
+#pragma unroll 4
+  for (; e < e1; e += step) {
+    const int c = idx[e];
+    const T a = val[e];
+    T x[Q];
+    ld_row<T, Q>(X + (size_t)c * Q, x);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) acc[k] = fma(a, x[k], acc[k]);
+  }
+}
+template <typename T, int Q, int JT, typename F>
+__device__ __noinline__ void spmm_long_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
+                                            const T* __restrict__ val, const T* X, int r0, int r1, int L, F row) {
+  __shared__ int nbig, big[ROW_BIG];
+  __shared__ T part[JT / 32][Q];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (tid == 0) nbig = 0;
+  __syncthreads();
+  T acc[Q];
+  auto warp_row = [&](int i, int e, int step) {
+#pragma unroll
+    for (int k = 0; k < Q; ++k) acc[k] = T(0);
+    spmm_add<T, Q>(idx, val, X, ptr[i] + e, ptr[i + 1], step, acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < Q; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+  };
+  for (int base = r0 + 32 * warp; base < r1; base += JT) {
+    const int mine = base + lane, len = mine < r1 ? ptr[mine + 1] - ptr[mine] : 0;
+    for (unsigned todo = __ballot_sync(0xffffffffu, len > ROW_LANE * L); todo; todo &= todo - 1) {
+      const int l = __ffs(todo) - 1, i = base + l;
+      if (__shfl_sync(0xffffffffu, len, l) > ROW_WARP) {
+        int at = lane == 0 ? atomicAdd(&nbig, 1) : 0;
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (at < ROW_BIG) {
+          if (lane == 0) big[at] = i;
+          continue;
+        }
+      }
+      warp_row(i, lane, 32);
+      if (lane == 0) row(i, acc);
+    }
+  }
+  __syncthreads();
+  for (int q = 0; q < min(nbig, ROW_BIG); ++q) {
+    const int i = big[q];
+    warp_row(i, tid, JT);
+    if (lane == 0)
+#pragma unroll
+      for (int k = 0; k < Q; ++k) part[warp][k] = acc[k];
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < JT / 32; ++w)
+#pragma unroll
+        for (int k = 0; k < Q; ++k) acc[k] += part[w][k];
+      row(i, acc);
+    }
+    __syncthreads();
+  }
+}
 template <typename T, int Q, int JT, typename F>
 __device__ __forceinline__ void spmm_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
                                           const T* __restrict__ val, const T* X, int r0, int r1, int L, F&& row) {
   const int per = JT / L, gl = threadIdx.x % L, gi = threadIdx.x / L;
+  bool any = false;
   for (int base = r0; base < r1; base += per) {   // uniform trip count: the shuffles need whole warps
     const int i = base + gi;
+    const int e0 = i < r1 ? ptr[i] : 0, e1 = i < r1 ? ptr[i + 1] : 0;
+    const bool later = e1 - e0 > ROW_LANE * L;
     T acc[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) acc[k] = T(0);
-    if (i < r1) {
-      const int e1 = ptr[i + 1];
-#pragma unroll 4
-      for (int e = ptr[i] + gl; e < e1; e += L) {
-        const int c = idx[e];
-        const T a = val[e];
-        T x[Q];
-        ld_row<T, Q>(X + (size_t)c * Q, x);
-#pragma unroll
-        for (int k = 0; k < Q; ++k) acc[k] = fma(a, x[k], acc[k]);
-      }
-    }
+    if (!later) spmm_add<T, Q>(idx, val, X, e0 + gl, e1, L, acc);
     for (int o = L / 2; o > 0; o >>= 1)
 #pragma unroll
       for (int k = 0; k < Q; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
-    if (i < r1 && gl == 0) row(i, acc);
+    if (i < r1 && gl == 0 && !later) row(i, acc);
+    any = any || later;
   }
+  if (__syncthreads_or(any)) spmm_long_rows<T, Q, JT>(ptr, idx, val, X, r0, r1, L, row);
 }
 
 // Lanes per row: as many as keep a row within a few rounds of gathers.

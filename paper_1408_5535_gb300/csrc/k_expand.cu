@@ -368,7 +368,7 @@ bool expand_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>& A
   // the line (above): in FP64 the cluster's arithmetic, in FP32 its reads of the
   // basis, and the product's gathers on 16 SMs against what the launches cost
   const double np = (double)n * (nlock + j + 8);
-  const double bytes = 2.0 * A.nnz * (Q + 2) * sizeof(T);
+  const double bytes = (A.skew + At.skew) * A.nnz * (Q + 2) * sizeof(T);
   if ((sizeof(T) == 8 ? np * (Q + 1) / 2e6 : np / 1e6) + bytes / (26e6 + 4e6 * Q) > 1.0) return false;
   ProfScope ps(s, sizeof(T) == 4 ? PROF_F32 + PROF_GRAM : PROF_GRAM);
   ExArgs g{};

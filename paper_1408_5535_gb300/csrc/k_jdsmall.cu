@@ -356,8 +356,9 @@ bool jd_solve_small(cudaStream_t s, const SparseView<T>& A, const SparseView<T>&
                     T* sol, T* cv, T* xrm, T* z, double* sc, int steps, double tol, int* done) {
   const int n = At.nrows, Q = q >= 5 ? 8 : q >= 3 ? 4 : q;
   // bytes a step moves through the cluster's L2 ports: Q (scaled form twice more),
-  // the vectors, the gathers
-  const double bytes = sizeof(T) * ((double)n * (nq * (scaled ? 4 : 2) + 20.0 * q) + 2.0 * A.nnz * (Q + 2));
+  // the vectors, the gathers (of the CTA with the most entries, times the CTAs)
+  const double bytes =
+      sizeof(T) * ((double)n * (nq * (scaled ? 4 : 2) + 20.0 * q) + (A.skew + At.skew) * A.nnz * (Q + 2));
   if (bytes > JD_SMALL_BYTES || nq > 64) return false;
   ProfScope ps(s, sizeof(T) == 4 ? PROF_F32 + PROF_SMALL : PROF_SMALL);
   JdArgs g{};

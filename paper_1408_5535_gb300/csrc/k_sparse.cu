@@ -560,7 +560,22 @@ void csr_to_csc(cudaStream_t s, int m, int n, int64_t nnz, const int* rp, const 
   else if (col <= 40.0)
     k_sort_cols<16><<<ceil_div((int64_t)n * 16, CSC_TH), CSC_TH, 0, s>>>(n, nnz, cp, va, ri, cv);
   else
-    k_sort_cols<32><<<ceil_div((int64_t)n * 32, CSC_TH), CSC_TH, 0, s>>>(n, cp, va, ri, cv);
+    k_sort_cols<32><<<ceil_div((int64_t)n * 32, CSC_TH), CSC_TH, 0, s>>>(n, nnz, cp, va, ri, cv);
+  count_launch();
+}
+
+__global__ void k_row_parts(int n1, const int* __restrict__ ptr1, int n2, const int* __restrict__ ptr2,
+                            int* __restrict__ out) {
+  const int m = threadIdx.x >> 5, r = threadIdx.x & 31;   // a warp per matrix
+  const int n = m ? n2 : n1, per = (n + ROW_PARTS - 1) / ROW_PARTS;
+  const int* ptr = m ? ptr2 : ptr1;
+  int v = 0;
+  if (r < ROW_PARTS) v = ptr[min((int64_t)n, (int64_t)(r + 1) * per)] - ptr[min((int64_t)n, (int64_t)r * per)];
+  v = __reduce_max_sync(0xffffffffu, v);
+  if (r == 0) out[m] = v;
+}
+void row_parts(cudaStream_t s, int n1, const int* ptr1, int n2, const int* ptr2, int* out) {
+  k_row_parts<<<1, 64, 0, s>>>(n1, ptr1, n2, ptr2, out);
   count_launch();
 }
 

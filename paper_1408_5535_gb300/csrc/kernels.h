@@ -35,10 +35,16 @@ struct SparseView {
   const int* ptr = nullptr;
   const int* idx = nullptr;
   const T* val = nullptr;
+  double skew = 1.0;   // entries of the fullest of ROW_PARTS equal parts of the rows, over their mean
   double avg_row() const { return nrows ? (double)nnz / nrows : 0.0; }
 };
 
 int lanes_for(double avg_row);
+
+// out[0], out[1] = entries of the fullest of ROW_PARTS equal parts of the rows of two matrices:
+// what a cluster of so many CTAs, each with its part, waits for.
+constexpr int ROW_PARTS = 16;
+void row_parts(cudaStream_t s, int n1, const int* ptr1, int n2, const int* ptr2, int* out);
 
 // Fixed-order reduction across thread blocks, so that repeated runs give the
 // same bits: block b stores its partial results at ws + b * (n1 + n2), and a

@@ -266,16 +266,21 @@ static void upload_matrix(phsvds_ctx* ctx, Pool& pool, DevA& d, int64_t m, int64
   d.cv = pool.get<double>(nnz);
   int* work = pool.get<int>(csc_work_ints(n));
   csr_to_csc(s, d.m, d.n, nnz, d.rp, d.ci, d.va, d.cp, d.ri, d.cv, work);
-  d.A64 = SparseView<double>{d.m, d.n, nnz, d.rp, d.ci, d.va};
-  d.At64 = SparseView<double>{d.n, d.m, nnz, d.cp, d.ri, d.cv};
+  row_parts(s, d.m, d.rp, d.n, d.cp, flags);
+  CUCHK(cudaMemcpyAsync(h.at<int>(0), flags, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  sync(s);
+  const double part = std::max<double>(1.0, (double)nnz / ROW_PARTS);
+  const double skew = std::max(1.0, h.at<int>(0)[0] / part), skew_t = std::max(1.0, h.at<int>(0)[1] / part);
+  d.A64 = SparseView<double>{d.m, d.n, nnz, d.rp, d.ci, d.va, skew};
+  d.At64 = SparseView<double>{d.n, d.m, nnz, d.cp, d.ri, d.cv, skew_t};
   d.Z64 = pool.get<double>((size_t)m * bmax);
   if (need32) {
     d.va32 = pool.get<float>(nnz);
     d.cv32 = pool.get<float>(nnz);
     to_float(s, nnz, d.va, d.va32);
     to_float(s, nnz, d.cv, d.cv32);
-    d.A32 = SparseView<float>{d.m, d.n, nnz, d.rp, d.ci, d.va32};
-    d.At32 = SparseView<float>{d.n, d.m, nnz, d.cp, d.ri, d.cv32};
+    d.A32 = SparseView<float>{d.m, d.n, nnz, d.rp, d.ci, d.va32, skew};
+    d.At32 = SparseView<float>{d.n, d.m, nnz, d.cp, d.ri, d.cv32, skew_t};
     d.Z32 = pool.get<float>((size_t)m * bmax);
   }
   if (need_diag) {
