@@ -94,8 +94,9 @@ typedef struct {
     uint64_t seed;         /* SplitMix64 seed of the random vectors the method draws */
     double time_limit_s;   /* 0 = none */
     int profile;           /* 1 = time kernel classes with CUDA events (stats.t_*_ms), default 0;
-                            * what otherwise runs as one launch over several classes then runs
-                            * as its separate kernels */
+                            * the append of a block of short vectors, one launch over several
+                            * classes otherwise, then runs as its separate kernels.  2 = stage 1's
+                            * projected eigensolve and inner solve as separate kernels as well */
     /* PHSVDS_PREC_LEARNED: host pointers, copied at the start of the solve.
      * learned_params: PHSVDS_CNN_NPARAM BF16 values; learned_features: 3 planes
      * of n floats (log diffusion, beta_x, beta_y per grid cell); the grid is

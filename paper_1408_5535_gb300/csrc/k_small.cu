@@ -3,7 +3,7 @@
 //    H = V^T W (the projected problem of GD+k in stage 1, Algorithm 2 step 7
 //    in stage 2), run in a warm frame (the working matrix A = S^T H S and the
 //    accumulated rotation S are kept between outer iterations): an FP32 pass
-//    followed by FP64 rotations (stage 2, and stage 1 under opts.profile), or FP64
+//    followed by FP64 rotations (stage 2, and stage 1 with opts.profile = 2), or FP64
 //    in one CTA or over an 8-CTA cluster (stage 1's default is in k_eig.cu);
 //  * the refined vector of stage 2 (Algorithm 2 step 8): the smallest right
 //    singular vector of the triangular factor R by inverse iteration, and the

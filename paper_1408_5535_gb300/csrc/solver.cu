@@ -443,8 +443,8 @@ static void frame_from_true(cudaStream_t s, int j, const double* Ht, double* S, 
   symmetrise(s, j, Aw, LD);
 }
 
-// Rayleigh-Ritz eigensolve of stage 2 (one target, the closest to tshift) and, where
-// the kernel classes are timed apart, of stage 1: an FP32
+// Rayleigh-Ritz eigensolve of stage 2 (one target, the closest to tshift) and, with
+// opts.profile = 2, of stage 1: an FP32
 // cyclic Jacobi pass does the large rotations of the warm frame (one SM's FP64
 // pipe is ~60x slower than its FP32 pipe), S <- S Sf is re-orthonormalised and
 // the exact FP64 frame S^T Ht S rebuilt, and an FP64 Jacobi pass, tight only on
@@ -838,7 +838,7 @@ struct Stage1 {
   unsigned char* outb;
   static constexpr int F0 = 912, FBAD = 40;   // flags' offset; the flag of a deferred check
   bool fuse = false;      // short vectors: one launch per block (k_expand.cu)
-  bool profile = false;
+  bool eig_apart = false;
   double* Sf = nullptr;
   // host state
   int j = 0, nlock = 0, nsp = 0, rand_ctr = 0;
@@ -895,10 +895,11 @@ struct Stage1 {
     cluster_eig = o.projected_solver != 1;
     eig_mode = o.projected_solver;
     graphs.enabled = !o.profile;  // the per-class timing events are not captured
-    // opts.profile times the kernel classes apart, opts.spmm names a schedule
-    profile = o.profile != 0;
+    // opts.profile times the kernel classes, so that what spans several of them (the append)
+    // is left apart, with 2 the projected eigensolve as well; opts.spmm names a schedule
+    eig_apart = o.profile >= 2;
     fuse = !o.profile && o.spmm == PHSVDS_SPMM_AUTO;
-    if (profile) Sf = pool.get<double>(LD * LD);
+    if (eig_apart) Sf = pool.get<double>(LD * LD);
     stag_window = std::max(100, 6 * (maxb - mins));
     const size_t nn = (size_t)n;
     V = pool.get<T>(nn * maxb);
@@ -1110,7 +1111,7 @@ struct Stage1 {
       // when the targets are resolvable in FP32, else FP64 Jacobi throughout
       // (GB300's FP64 latency is ~14x its FP32 latency)
       const bool mixed_eig = !bmode && eig_mode == 2 && (largest || eig32_ok);
-      const bool one_eig = mixed_eig && !profile;   // opts.profile: its kernels apart
+      const bool one_eig = mixed_eig && !eig_apart;
       const bool pending = nb > 0 && expand(nb, one_eig);
       const int ntg = bmode ? 0 : std::min(b, k - nlock) + 1;   // B: every pair to the tight threshold
       const int omode = bmode ? 3 : (largest ? 1 : 0);
@@ -2186,7 +2187,7 @@ static void solve_impl(phsvds_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const
       op32 = tuned_spmm<float>(ctx, pool, A.A32, A.At32, A.Z32, A.n, spmm_width(b), &cached32, o.deterministic);
   }
   const int sch64 = op64.schedule;
-  const bool fuse = !o.profile && o.spmm == PHSVDS_SPMM_AUTO;
+  const bool fuse = o.profile < 2 && o.spmm == PHSVDS_SPMM_AUTO;   // the inner solve
   if (st) {
     std::memset(st, 0, sizeof(*st));
     st->spmm_schedule = sch64;
