@@ -670,16 +670,23 @@ CLASS_NAMES = ["fused A^T A SpMM (FP64)", "Gram / CGS passes (FP64)", "basis tra
                "projected eigensolvers (Jacobi)",
                "fused A^T A SpMM (FP32)", "Gram / CGS passes (FP32)", "basis transforms / Ritz vectors (FP32)",
                "inner MINRES vector kernels (FP32)", "A / A^T products (FP32)", "(unused FP32 Jacobi)"]
-CLASS_KERNELS = {0: "k_csr_rows / k_ata_fused <double>", 1: "k_cgs_pass<double>", 2: "k_tall_small<double>",
+CLASS_KERNELS = {0: "k_csr_rows / k_ata_fused <double>", 1: "k_cgs_split / k_cgs_pass<double>",
+                 2: "k_tall_rows / k_tall_cols / k_tall_stream<double> / k_tall_small",
                  4: "k_csr_rows<double, 1>", 6: "k_csr_rows / k_ata_fused <float>", 7: "k_cgs_pass<float>",
-                 8: "k_tall_small<float>", 9: "k_jd_lanczos / k_jd_update / k_col_dots", 10: "k_csr_rows<float, 1>"}
+                 8: "k_tall_stream<float>", 9: "k_jd_lanczos / k_jd_update / k_col_dots", 10: "k_csr_rows<float, 1>"}
 
 
-# the stage-1 projected eigensolve of a call: the FP32 pass and the FP64
+# the projected eigensolve of stage 1 (k_eig.cu, one launch)
+EIG_FUNCS = ["dot_col", "rsqrt_fast", "rcp_fast", "k_eig_step"]
+# its separate kernels (opts.profile = 2): the FP32 pass and the FP64
 # clean-up of the target pairs, with the device helpers they call
 JACOBI_FUNCS = ["rr_pair", "rot_params", "rot_params_small", "k_jacobi_eig", "k_jacobi_targets"]
-# the block Gram-Schmidt pass (its ncu capture: profiles/cgs_pass_f64_1e6x5e5.txt)
+# the block Gram-Schmidt pass: FP32 (its ncu capture: profiles/cgs_pass_f32_1e6x5e5.txt), and FP64
+# as digit products (profiles/cgs_split_f64_1e6x5e5.txt)
+CGS_FILES = ["k_tall.cu", "common.cuh"]
 CGS_FUNCS = ["cp_async16", "cp_async_wait_all", "stage_cols", "lds_vec", "reduce_scatter_step", "k_cgs_pass"]
+CGS_SPLIT_FUNCS = ["fix62", "pack_digits", "mma16", "redo_list", "coeff_scales", "row_scales", "rows_times_coeff",
+                   "col_scale", "k_cgs_split"]
 # the row kernel of the two-phase SpMM (its capture: profiles/spmm_csr_rows_c3_f32.txt)
 SPMM_FUNCS = ["load_row_256", "l2_evict_first_policy", "ld_stream", "gather_rows", "load_slots", "k_csr_rows"]
 SPMM_FUSED_FUNCS = ["load_row_256", "l2_evict_first_policy", "ld_stream", "gather_rows", "load_slots",
@@ -687,13 +694,15 @@ SPMM_FUSED_FUNCS = ["load_row_256", "l2_evict_first_policy", "ld_stream", "gathe
 
 
 def kernel_source_sha256(kernel_file, names):
-    """sha256 of the source text of the named functions of a .cu file (each
-    from the line that declares it to its closing brace in column 0, every
-    overload), so that edits elsewhere in the file do not invalidate a
-    capture."""
+    """sha256 of the source text of the named functions of a .cu file, or of a
+    list of files (each from the line that declares it to its closing brace in
+    column 0, every overload), so that edits elsewhere in the file do not
+    invalidate a capture."""
     import hashlib
+    lines = []
     try:
-        lines = open(os.path.join(ROOT, "paper_1408_5535_gb300", "csrc", kernel_file)).read().splitlines()
+        for f in [kernel_file] if isinstance(kernel_file, str) else kernel_file:
+            lines += open(os.path.join(ROOT, "paper_1408_5535_gb300", "csrc", f)).read().splitlines()
     except OSError:
         return None
     h = hashlib.sha256()
@@ -751,8 +760,8 @@ def roofline_for(A, prof, dom, hbm, peak_kind):
         flops = 18.0 * j_avg * rot
         per_call_ms = t_ms / jc
         ach = flops / (per_call_ms * 1e-3) / 1e9
-        tr = measured_traffic("k_small.cu", JACOBI_FUNCS, "jacobi_fp32_targets_grid32.txt", "dram_bytes_per_call")
-        return {"bound": "alu", "kernel": "stage-1 projected eigensolve (Jacobi kernels of k_small.cu)",
+        tr = measured_traffic("k_eig.cu", EIG_FUNCS, "eig_step_f64.txt", "dram_bytes_per_launch")
+        return {"bound": "alu", "kernel": "stage-1 projected eigensolve (k_eig_step: FP32 Jacobi, FP64 refinement)",
                 "achieved": ach / 1e3, "peak": FP64_PEAK_GFLOPS / 1e3, "unit": "TFLOP/s",
                 "frac": ach / FP64_PEAK_GFLOPS, "traffic": tr,
                 "peak_source": "nominal FP64 rate of the GPU (152 SMs x 2 FMA/clk)",
@@ -765,8 +774,9 @@ def roofline_for(A, prof, dom, hbm, peak_kind):
            "flops_per_launch": fl / calls if calls else None, "bytes_per_launch": by / calls if calls else None,
            "traffic": None}
     if dom in (1, 7):
-        out["traffic"] = measured_traffic("k_tall.cu", CGS_FUNCS, "cgs_pass_%s_1e6x5e5.txt" % ("f64" if dom == 1 else "f32"),
-                                          "dram_bytes_per_launch")
+        out["traffic"] = (measured_traffic("k_split.cu", CGS_SPLIT_FUNCS, "cgs_split_f64_1e6x5e5.txt",
+                                           "dram_bytes_per_launch") if dom == 1 else
+                          measured_traffic(CGS_FILES, CGS_FUNCS, "cgs_pass_f32_1e6x5e5.txt", "dram_bytes_per_launch"))
         if out["traffic"] is not None:
             out["traffic_launch"] = ("the captured launch: n = 500,000, p = 55 basis columns, q = 8, "
                                      "Gsub and Gout (profiles/)")
@@ -786,6 +796,9 @@ def roofline_for(A, prof, dom, hbm, peak_kind):
         out.update(bound="alu", achieved=ach, peak=FP64_PEAK_GFLOPS / 1e3, unit="TFLOP/s",
                    frac=(ach * 1e3 / FP64_PEAK_GFLOPS) if ach else None,
                    peak_source="nominal FP64 rate of the GPU (152 SMs x 2 FMA/clk x 2.06 GHz)")
+        if dom in (1, 2):
+            out["note"] = ("the products of long vectors run as digit products on the FP16 tensor cores (k_split.cu): "
+                           "their rate is above the FP64 pipe's")
     else:
         ach = by / (t_ms * 1e-3) / 1e9 if t_ms else None
         out.update(bound="hbm", achieved=ach, peak=hbm, unit="GB/s", frac=(ach / hbm) if ach else None,

@@ -98,3 +98,13 @@ def test_oracle_samples_are_scaled_by_the_recorded_iterations():
     assert gold and total == gi and est == pytest.approx(10.0 / 5 * gi) and v == pytest.approx(20 / est)
     v, est, total, gold = bench._scaled(ns, 20, {"seconds": 10.0, "iters": 5, "finished": True}, 999)
     assert est == 10.0
+
+
+def test_captures_of_the_dominant_classes_match_the_source():
+    """The Gram-Schmidt passes and the projected eigensolve: the committed ncu summaries are of the
+    kernels as they are, also where a helper lives in another file."""
+    assert bench.measured_traffic(bench.CGS_FILES, bench.CGS_FUNCS, "cgs_pass_f32_1e6x5e5.txt",
+                                  "dram_bytes_per_launch") == 133099008.0
+    assert bench.measured_traffic("k_split.cu", bench.CGS_SPLIT_FUNCS, "cgs_split_f64_1e6x5e5.txt",
+                                  "dram_bytes_per_launch") > 2e8
+    assert bench.measured_traffic("k_eig.cu", bench.EIG_FUNCS, "eig_step_f64.txt", "dram_bytes_per_launch") > 0
