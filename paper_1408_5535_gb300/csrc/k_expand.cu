@@ -17,18 +17,21 @@
 // across CTAs; in FP64 plainly.
 //
 // Time per iteration of stage 1 with the general form and with this one (2n x n, 8 entries
-// per row, 35 basis vectors at most, blocks of 1, 4, 8):
-//   FP64 n =  1000   202 138   350 253   496 359 us
-//        n =  4000   206 150   347 288   488 418
-//        n =  8000   215 171   355 344   541 566
-//        n = 16000   226 214   370 479
-//        n = 32000   245 296
-//   FP32 n =  1000   196 129   312 205   441 294
-//        n = 16000   216 177   348 271   527 418
-//        n = 32000   217 227   359 334   554 528
-//        n = 64000   234 319   389 444   518 567
+// per row, 35 basis vectors at most, blocks of 1, 4, 8); a dash: this one not taken (forced, it
+// was the slower one there):
+//   FP64 n =   300   212 144   406 304   641 469 us
+//        n =  1000   210 144   360 272   507 387
+//        n =  2000   207 151   356 309   521 455
+//        n =  8000   225 175   365 350   553  -
+//        n = 16000   232 223   380  -    566  -
+//   FP32 n =   300   200 129   337 218   521 348
+//        n =  1000   207 133   335 218   461 313
+//        n =  8000   219 156   339 248   487 370
+//        n = 16000   230 186   366 290   541 451
+//        n = 32000   227  -    375  -    568  -
 // In FP64 the 16 SMs' arithmetic decides (n p b), in FP32 their reads of the basis
-// (n p).  A 2000 x 1000 solve with the defaults: 174 ms -> 121 ms.
+// (n p).  A 2000 x 1000 solve with the defaults: 174 ms -> 122 to 140 ms (its iterations vary
+// with the autotuned product).
 #include <algorithm>
 
 #include <cooperative_groups.h>
@@ -351,7 +354,10 @@ bool go(cudaStream_t s, ExArgs g) {
   g.cap = ((std::max(g.nlock + g.j, g.j + g.nb) + Q) * Q + 1) & ~1;
   g.nc = cluster_size(k_expand_cluster<T, Q>, XT, SMEM_MAX, SMEM_MAX, known);
   if (g.nc == 0) return false;
-  if (g.n <= 2048) g.nc = 8;                       // as fast as 16 at n = 1000 (143 us per iteration both)
+  // 8 leave half of the SMs to the other solves of a batch, and take as long for one vector (per
+  // iteration at n = 300, 500, 1000: 144, 148, 144 us with either; blocks of 8 at n = 2000: 455,
+  // with 16 440)
+  if (g.n <= 2048) g.nc = 8;
   g.rows = ((g.n + g.nc - 1) / g.nc + 1) & ~1;
   const size_t smem = expand_smem(g.nc, g.cap, Q, g.rows, sizeof(T));
   if (smem > SMEM_MAX) return false;

@@ -14,8 +14,9 @@
 //   4. y = A^T z (own rows), Q^T y, u^T y, u^T u, x^T y
 //   5. the projected, shifted operator and the Lanczos recurrence, ||y||^2
 //   6. Givens step, w, s, v (no barrier: own rows)
-// One cluster has the bandwidth of 16 SMs, about 0.35 TB/s of L2, and a step has 5
-// or 7 barriers of 2 to 3 us with their ramps.  Time of stage 1 per step, general
+// One cluster has the bandwidth of 16 SMs, about 0.35 TB/s of L2, and a step has 4
+// barriers, in the scaled form 5 (after xrm, z and each reduction), at 4 to 6 us with the
+// work between them (29 us at n = 4096).  Time of stage 1 per step, general
 // form and this one (four systems, scaled form, weighted grid gradients):
 //   n = 4096 FP32 (3 MB moved)      71 and 29 us    n = 10,000 FP64 (15 MB) 112 and 83 us
 //   n = 16,384 FP64 (24 MB)        114 and 94 us    n = 32,400 FP32 (24 MB)  84 and 68 us

@@ -46,6 +46,7 @@
 //
 // A tile with an Inf, a NaN or values below 2^-950 is computed in plain FP64.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -647,7 +648,8 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
       Acc acc;
       Mag mag;
       rows_times_coeff<KT, TS_LD, ST>(buf, sc, set, Bs, g, t, lane, base, acc, mag);
-      const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
+      const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW);
+      const unsigned l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
       // what the kept-out coefficient of output q's column multiplies
       auto x_of = [&](int q) { return buf[sc.peak[c0 + (q & 1)] * TS_LD + g + (q < 2 ? 0 : 8)]; };
       auto finish = [&](int q, double o) {
@@ -665,7 +667,8 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const int c = c0 + (q & 1);
-            if (sc.peak[c] >= 0 && peak_holds(x_of(q), sc.ypeak[c], base[q < 2 ? 0 : 1], sc.F[set][c])) need &= ~(1u << q);
+            if (sc.peak[c] >= 0 && peak_holds(x_of(q), sc.ypeak[c], base[q < 2 ? 0 : 1], sc.F[set][c]))
+              need &= ~(1u << q);
           }
         }
         if (__any_sync(0xffffffffu, need)) {
@@ -836,7 +839,8 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
             const unsigned need = (weak >> (16 * h + 4 * j)) & 15u;
             if (!__any_sync(0xffffffffu, need)) continue;
             double fix[4];
-            most = max(most, redo_list(need, Y + (size_t)j * 16 * ldy, ldy, 1, buf + 8 * h, 1, TS_LD, p, list[warp], fix));
+            most = max(most, redo_list(need, Y + (size_t)j * 16 * ldy, ldy, 1, buf + 8 * h, 1, TS_LD, p, list[warp],
+                                       fix));
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               if (!((need >> q) & 1u)) continue;
@@ -972,7 +976,8 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
         Mag mag;
         rows_times_coeff<KT, CS_LD, ST>(cur, sc, set, Bs, g, t, lane, base, acc, mag);
         const int i0 = row0 + 16 * warp + g;       // (rows past n are zero)
-        const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW), l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
+        const unsigned l0 = mag.levels(0) | pad | (i0 < n ? 0u : NO_ROW);
+        const unsigned l1 = mag.levels(1) | pad | (i0 + 8 < n ? 0u : NO_ROW);
         double out[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -1051,8 +1056,9 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
           }
           const int s0 = te[ch][2 * t], s1 = te[ch][2 * t + 1];
           const unsigned s01 = (unsigned)s0 | (unsigned)s1 << 16;
-          const unsigned w0 = raise(e0 * 0x10001u + s01, mag.levels(0) | pad | (16 * m + g < p ? 0u : NO_ROW), gtop[0]);
-          const unsigned w1 = raise(e1 * 0x10001u + s01, mag.levels(1) | pad | (16 * m + g + 8 < p ? 0u : NO_ROW), gtop[1]);
+          const unsigned l0 = mag.levels(0) | pad | (16 * m + g < p ? 0u : NO_ROW);
+          const unsigned l1 = mag.levels(1) | pad | (16 * m + g + 8 < p ? 0u : NO_ROW);
+          const unsigned w0 = raise(e0 * 0x10001u + s01, l0, gtop[0]), w1 = raise(e1 * 0x10001u + s01, l1, gtop[1]);
           double out[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i)
@@ -1096,7 +1102,8 @@ __global__ void __launch_bounds__(CS_W * 32, 2)
             }
           }
           const int e = te[tch][g], s0 = e + te[tch][2 * t], s1 = e + te[tch][2 * t + 1];
-          const unsigned w = raise((unsigned)s0 | (unsigned)s1 << 16, mag.levels(0) | pad | (g < q ? 0u : NO_ROW), ttop);
+          const unsigned l0 = mag.levels(0) | pad | (g < q ? 0u : NO_ROW);
+          const unsigned w = raise((unsigned)s0 | (unsigned)s1 << 16, l0, ttop);
           double out[4] = {times_pow2(acc.sum(0), s0 - E_OUT), times_pow2(acc.sum(1), s1 - E_OUT), 0.0, 0.0};
           if (ST && any_less2(ttop, w) && row0 + tch * RC < n)
             redo(less2(ttop, w), Ts + tch * RC, CS_LD, 1, Ts + tch * RC, CS_LD, 1, RC, list[warp], out);
@@ -1163,11 +1170,12 @@ void tall_go(cudaStream_t s, int n, const double* P, int ldp, int p, const doubl
   const int grid = std::min(split_sms(), ceil_div(n, TS_R));
   const RedWs rw = norms2 ? red_ws((size_t)grid * r) : RedWs{};
   if (r <= 8)
-    k_tall_rows<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
-                                                      even16(P, ldp), sm.tiles, rw);
+    k_tall_rows<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta,
+                                                                    norms2, even16(P, ldp), sm.tiles, rw);
   else
-    k_tall_cols<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2,
-                                                      even16(P, ldp), even16(Out, ldo), sm.tiles, sm.norms, rw);
+    k_tall_cols<KT, ST><<<grid, tall_warps(KT) * 32, sm.total, s>>>(n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta,
+                                                                    norms2, even16(P, ldp), even16(Out, ldo), sm.tiles,
+                                                                    sm.norms, rw);
   count_launch();
   if (norms2) reduce_partials(s, rw, grid, r, norms2, 0, nullptr);
 }
@@ -1201,11 +1209,14 @@ bool tall_split(cudaStream_t s, int n, const double* P, int ldp, int p, const do
   if (n < 512 || n > INT32_MAX - 256 || r < 3 || p < 8 || p > 64 || r > 64 ||
       TallSmem(KT, r, norms2 != nullptr).total > SPLIT_SMEM)
     return false;
+  auto go = [&](auto kt) {
+    (strict ? tall_go<kt(), true> : tall_go<kt(), false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2);
+  };
   switch (KT) {
-    case 1: (strict ? tall_go<1, true> : tall_go<1, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    case 2: (strict ? tall_go<2, true> : tall_go<2, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    case 3: (strict ? tall_go<3, true> : tall_go<3, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
-    default: (strict ? tall_go<4, true> : tall_go<4, false>)(s, n, P, ldp, p, Y, ldy, r, Out, ldo, Xs, ldx, theta, norms2); break;
+    case 1: go(std::integral_constant<int, 1>()); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 3: go(std::integral_constant<int, 3>()); break;
+    default: go(std::integral_constant<int, 4>()); break;
   }
   return true;
 }
@@ -1221,11 +1232,14 @@ bool cgs_split(cudaStream_t s, int n, const Basis<double>& P, double* Tb, int ld
   if (n < (q >= 5 ? 512 : 8192) || n > INT32_MAX - 256 || q < 3 || p < (q >= 5 ? 10 : 16) || p > 64 ||
       !(Gsub || Gout))
     return false;
+  auto go = [&](auto kt) {
+    (strict ? cgs_go<kt(), true> : cgs_go<kt(), false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout);
+  };
   switch ((p + 15) / 16) {
-    case 1: (strict ? cgs_go<1, true> : cgs_go<1, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    case 2: (strict ? cgs_go<2, true> : cgs_go<2, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    case 3: (strict ? cgs_go<3, true> : cgs_go<3, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
-    default: (strict ? cgs_go<4, true> : cgs_go<4, false>)(s, n, P, Tb, ldt, q, Gsub, Gout, Tout); break;
+    case 1: go(std::integral_constant<int, 1>()); break;
+    case 2: go(std::integral_constant<int, 2>()); break;
+    case 3: go(std::integral_constant<int, 3>()); break;
+    default: go(std::integral_constant<int, 4>()); break;
   }
   return true;
 }

@@ -402,10 +402,10 @@ static void tall_general(cudaStream_t s, int n, const double* P, int ldp, int p,
 // memory.  Each basis value is used by one thread only, so staging it would
 // only add a barrier per chunk.  Several rows share a broadcast; with few rows,
 // one per thread spreads them over more SMs.  The norms are summed per thread
-// and reduced once, at the end.  Bound by HBM in FP32 (by latency towards wide
-// outputs, whose sums leave few warps) and by the FP64 pipe in FP64.  Measured
+// and reduced once, at the end.  Bound by latency and issue in FP32 (one wave of one
+// streaming pass; 23% of HBM at 155,649 rows) and by the FP64 pipe in FP64.  Measured
 // against staging with a butterfly per norm: FP32, 155,649 rows, 35 columns to
-// 8 with norms, 46 us -> 19 us (1.6 TB/s; 10 us without norms); 500,000 rows, 35
+// 8 with norms, 46 us -> 20 us (1.55 TB/s; 10 us without norms); 500,000 rows, 35
 // columns to 21, 60 us -> 42 us; FP64, 500,000 rows, 35 columns to 1, 256 us ->
 // 37 us (a staged result takes the FP64 work of 8 columns).
 constexpr int ST_TH = 128;

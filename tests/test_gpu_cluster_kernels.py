@@ -150,7 +150,8 @@ def test_append_sums_of_equal_terms_in_fp32(lib, n):
 @pytest.mark.parametrize("dt,tol,lim", [(np.float64, 1e-9, 1e-8), (np.float32, 1e-3, 5e-3)], ids=["f64", "f32"])
 @pytest.mark.parametrize("scaled", [False, True])
 @pytest.mark.parametrize("m,n,q,nl,long_rows", [(40, 30, 1, 0, []), (700, 600, 3, 4, []), (900, 777, 5, 0, [65, 700]),
-                                                (3000, 2600, 8, 6, [64, 2600]), (2200, 2100, 7, 1, []), (5100, 5000, 2, 3, [5000])])
+                                                (3000, 2600, 8, 6, [64, 2600]), (2200, 2100, 7, 1, []),
+                                                (5100, 5000, 2, 3, [5000])])
 def test_inner_solve(lib, dt, tol, lim, scaled, m, n, q, nl, long_rows):
     """Every column solves its projected, shifted equation to the tolerance (the recursion's own
     residual, so a few times it is allowed)."""
@@ -195,7 +196,8 @@ def test_inner_solve(lib, dt, tol, lim, scaled, m, n, q, nl, long_rows):
     v[:q] = _dev((R / b1[:q]).T, dt)
     xrm, z = (torch.full((k, 8), 7.0, dtype=tt, device="cuda") for k in (n, m))
     done = torch.zeros(1, dtype=torch.int32, device="cuda")
-    dq, dx, dd, dth, dsc = _dev(Q.T if Q.shape[1] else np.zeros((1, n)), dt), _dev(X.T, dt), _dev(ds, dt), _dev(theta, np.float64), _dev(sc, np.float64)
+    dq, dx, dd = (_dev(M, dt) for M in (Q.T if Q.shape[1] else np.zeros((1, n)), X.T, ds))
+    dth, dsc = _dev(theta, np.float64), _dev(sc, np.float64)
     null = C.c_void_p(0)
     ok = _call(lib, SOLVE % ("f" if dt == np.float32 else "d"),
                [A, At, q, Q.shape[1], C.c_bool(scaled), dq, null if scaled else dx, dd if scaled else null, dth, v,
