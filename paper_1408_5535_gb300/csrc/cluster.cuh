@@ -106,11 +106,18 @@ __device__ __noinline__ void spmm_long_rows(const int* __restrict__ ptr, const i
     __syncthreads();
   }
 }
+// Whether rows [r0, r1) hold such a long one (for the whole CTA; a barrier).
+template <int JT>
+__device__ inline bool long_rows(const int* __restrict__ ptr, int r0, int r1, int L) {
+  bool any = false;
+  for (int i = r0 + threadIdx.x; i < r1; i += JT) any = any || ptr[i + 1] - ptr[i] > ROW_LANE * L;
+  return __syncthreads_or(any);
+}
 template <typename T, int Q, int JT, typename F>
 __device__ __forceinline__ void spmm_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
-                                          const T* __restrict__ val, const T* X, int r0, int r1, int L, F&& row) {
+                                          const T* __restrict__ val, const T* X, int r0, int r1, int L, bool any_long,
+                                          F&& row) {
   const int per = JT / L, gl = threadIdx.x % L, gi = threadIdx.x / L;
-  bool any = false;
   for (int base = r0; base < r1; base += per) {   // uniform trip count: the shuffles need whole warps
     const int i = base + gi;
     const int e0 = i < r1 ? ptr[i] : 0, e1 = i < r1 ? ptr[i + 1] : 0;
@@ -123,9 +130,8 @@ __device__ __forceinline__ void spmm_rows(const int* __restrict__ ptr, const int
 #pragma unroll
       for (int k = 0; k < Q; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
     if (i < r1 && gl == 0 && !later) row(i, acc);
-    any = any || later;
   }
-  if (__syncthreads_or(any)) spmm_long_rows<T, Q, JT>(ptr, idx, val, X, r0, r1, L, row);
+  if (any_long) spmm_long_rows<T, Q, JT>(ptr, idx, val, X, r0, r1, L, row);
 }
 
 // Lanes per row: as many as keep a row within a few rounds of gathers.

@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(XT, 1) k_expand_cluster(ExArgs g) {
     const int c = e / R, i = e - c * R;
     ts[e] = c < q && i < nr ? Tb[(size_t)c * n + i] : T(0);
   }
+  const bool long_a = long_rows<XT>(g.rp, m0, m1, g.la), long_t = long_rows<XT>(g.cp, i0, i0 + nr, g.lat);
   cl.sync();                                       // (every CTA has started: its shared memory can be written)
   int par = 0;
   // sum[l * Q + r] = sum over all rows of (column l) . T(:, r): the columns of Xl
@@ -316,10 +317,11 @@ __global__ void __launch_bounds__(XT, 1) k_expand_cluster(ExArgs g) {
   }
   scale(true);
   cl.sync();
-  spmm_rows<T, Q, XT>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la,
+  spmm_rows<T, Q, XT>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la, long_a,
                       [&](int i, const T (&acc)[Q]) { store_row<T, Q>(z + (size_t)i * Q, acc); });
   cl.sync();
-  spmm_rows<T, Q, XT>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i0 + nr, g.lat, [&](int i, const T (&acc)[Q]) {
+  spmm_rows<T, Q, XT>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i0 + nr, g.lat, long_t,
+                      [&](int i, const T (&acc)[Q]) {
 #pragma unroll
     for (int c = 0; c < Q; ++c) {
       ts[c * R + i - i0] = acc[c];

@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(JT, 1) k_jd_cluster(JdArgs g) {
     sm.cf[0][c] = (T)sm.theta[c];
     sm.cf[8][c] = sm.act[c] != 0.0 ? T(1) : T(0);
   }
+  const bool long_a = long_rows<JT>(g.rp, m0, m1, g.la), long_t = long_rows<JT>(g.cp, i0, i1, g.lat);
   cl.sync();                                       // every CTA has started, and its scalars are set
   int par = 0;                                     // parity of the reductions
   // sm.sum / sm.sumt[0 .. cnt) = the sums over the CTAs of sm.wsum
@@ -188,11 +189,11 @@ __global__ void __launch_bounds__(JT, 1) k_jd_cluster(JdArgs g) {
     }
     cl.sync();
     // ---- 3: z = A u
-    spmm_rows<T, Q, JT>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la,
+    spmm_rows<T, Q, JT>(g.rp, g.ci, static_cast<const T*>(g.va), xrm, m0, m1, g.la, long_a,
                     [&](int i, const T (&acc)[Q]) { store_row<T, Q>(z + (size_t)i * Q, acc); });
     cl.sync();
     // ---- 4: y = A^T z on the own rows, and its projections
-    spmm_rows<T, Q, JT>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i1, g.lat, [&](int i, const T (&acc)[Q]) {
+    spmm_rows<T, Q, JT>(g.cp, g.ri, static_cast<const T*>(g.cv), z, i0, i1, g.lat, long_t, [&](int i, const T (&acc)[Q]) {
 #pragma unroll
       for (int c = 0; c < Q; ++c)
         if (c < q) cv[(size_t)c * n + i] = acc[c];

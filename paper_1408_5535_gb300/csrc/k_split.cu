@@ -347,26 +347,25 @@ __device__ inline void coeff_scales(const double* __restrict__ Y, int ldy, int p
   const int warp = tid >> 5, lane = tid & 31;
   for (int c = warp; c < rc; c += NT / 32) {
     int f0 = 0, f1 = -4096, inf = 0, nz = 0, peak = -1;
+    double y[2];                                 // (p <= 64)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) y[u] = lane + 32 * u < p && c < r ? Y[lane + 32 * u + (size_t)c * ldy] : 0.0;
     if (PEAK && c < r) {
-      unsigned m0 = 0, m1 = 0;                   // the lane's larger and smaller, by their high words
-      int k0 = -1;
-      for (int k = lane; k < p; k += 32) {
-        const unsigned m = (unsigned)__double2hiint(Y[k + (size_t)c * ldy]) & 0x7fffffffu;
-        m1 = max(m1, min(m, m0));
-        if (m >= m0) k0 = k;
-        m0 = max(m0, m);
-      }
+      // the lane's larger and smaller, by their high words
+      const unsigned ma = (unsigned)__double2hiint(y[0]) & 0x7fffffffu;
+      const unsigned mb = (unsigned)__double2hiint(y[1]) & 0x7fffffffu;
+      const unsigned m0 = max(ma, mb), m1 = min(ma, mb);
       const unsigned top = __reduce_max_sync(0xffffffffu, m0);
       const int at = __ffs(__ballot_sync(0xffffffffu, m0 == top)) - 1;
       const unsigned next = __reduce_max_sync(0xffffffffu, lane == at ? m1 : m0);
-      peak = __shfl_sync(0xffffffffu, k0, at);
+      peak = __shfl_sync(0xffffffffu, mb > ma ? lane + 32 : lane, at);
       if (top < next + (3u << 20)) peak = -1;
     }
-    for (int k = lane; k < p && c < r; k += 32) {
-      const double y = Y[k + (size_t)c * ldy];
-      const int e = expo(y);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int k = lane + 32 * u, e = expo(y[u]);
       inf |= e == 0x7ff;
-      if (y == 0.0 || k == peak) continue;
+      if (y[u] == 0.0 || k == peak) continue;
       nz = 1;
       f0 = max(f0, e);
       f1 = max(f1, e + sc.b[1][k]);
@@ -375,6 +374,7 @@ __device__ inline void coeff_scales(const double* __restrict__ Y, int ldy, int p
     f1 = __reduce_max_sync(0xffffffffu, f1);
     inf = __any_sync(0xffffffffu, inf);
     nz = __any_sync(0xffffffffu, nz);
+    const double ypeak = __shfl_sync(0xffffffffu, peak >= 32 ? y[1] : y[0], peak & 31);
     if (lane == 0) {
       if (inf || (nz && f0 < E_MIN)) sc.bad = 1;
       if (nz) {
@@ -384,7 +384,7 @@ __device__ inline void coeff_scales(const double* __restrict__ Y, int ldy, int p
       sc.peak[c] = peak;
       if (peak >= 0) {
         sc.peaks = 1;
-        sc.ypeak[c] = Y[peak + (size_t)c * ldy];
+        sc.ypeak[c] = ypeak;
       }
       sc.F[0][c] = max(f0, E_MIN);
       sc.F[1][c] = max(f1, E_MIN);
