@@ -55,8 +55,9 @@ __device__ __forceinline__ void spmm_add(const int* __restrict__ idx, const T* _
     for (int k = 0; k < Q; ++k) acc[k] = fma(a, x[k], acc[k]);
   }
 }
+// (In line: a call, though never made, costs every step of an inner solve 0.5 us of 28.)
 template <typename T, int Q, int JT, typename F>
-__device__ __noinline__ void spmm_long_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
+__device__ __forceinline__ void spmm_long_rows(const int* __restrict__ ptr, const int* __restrict__ idx,
                                             const T* __restrict__ val, const T* X, int r0, int r1, int L, F row) {
   __shared__ int nbig, big[ROW_BIG];
   __shared__ T part[JT / 32][Q];
