@@ -40,7 +40,7 @@
 //
 // Measured on the FP64 pipe and here: Gram-Schmidt pass, 500,000 x 55 against 8,
 // subtract and project, 796 us -> 225 us; V Y, 500,000 x 35 to 21, 694 us -> 173 us; to
-// 8, 265 us -> 79 us (without the sums of moduli 218, 173 and 74 us).  Where outputs are
+// 8, 265 us -> 81 us (without the sums of moduli 218, 173 and 74 us).  Where outputs are
 // computed anew it takes longer: the pass on log-normal(2) elements 542 us, on elements over 10
 // decades 705 us; V Y of such up to 850 us.
 //
@@ -684,7 +684,7 @@ __global__ void __launch_bounds__(tall_warps(KT) * 32, 1)
         if (next < ntiles) load_cols<TS_R, TS_LD, 32>(P, ldp, p, n, next * TS_R, vec, buf, lane);
         cp_commit();
       };
-      if (!ST || !sc.peaks) reload();                   // beside the sums (79 us; after them 87)
+      if (!ST || !sc.peaks) reload();                   // beside the sums (81 us; after them 87)
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int c = c0 + (q & 1);

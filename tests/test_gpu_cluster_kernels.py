@@ -252,3 +252,40 @@ def test_projected_eigensolve(lib, kind, j, ntarget, ident, largest):
     assert np.max(np.abs(t[o[: min(ntarget, j)]] - ref[: min(ntarget, j)])) <= 32 * eps * nH
     assert np.array_equal(sc.cpu().numpy().T[:j, :nt], S[:, o[:nt]]) and np.array_equal(thc.cpu().numpy()[:nt], t[o[:nt]])
     assert nrm.cpu().numpy()[:nt].max() == 0.0
+
+
+@pytest.mark.parametrize("n1,n2", [(1, 1), (15, 16), (17, 33), (1000, 4097), (5, 100000)])
+def test_entries_of_the_fullest_part_of_the_rows(lib, n1, n2):
+    rng = np.random.default_rng(n2)
+    ptrs, ref = [], []
+    for n in (n1, n2):
+        rp = np.concatenate([[0], np.cumsum(rng.poisson(3.0, n) * (rng.random(n) < 0.2) * 9)]).astype(np.int64)
+        per = -(-n // 16)
+        ref.append(max(rp[min(n, (r + 1) * per)] - rp[min(n, r * per)] for r in range(16)))
+        ptrs.append(_dev(rp, np.int32))
+    out = torch.full((2,), -1, dtype=torch.int32, device="cuda")
+    _call(lib, "_ZN2ph9row_partsEP11CUstream_stiPKiiS3_Pi", [n1, ptrs[0], n2, ptrs[1], out], None)
+    assert out.tolist() == ref
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64], ids=["f32", "f64"])
+def test_append_is_left_to_the_general_form_where_one_part_holds_the_entries(lib, dt):
+    """The same sizes with the entries spread (taken) and more and more of them in one sixteenth of
+    the rows of A and A^T: the line counts that part, as if all were as full."""
+    rng = np.random.default_rng(1)
+    n = 4000
+    S = _matrix(rng, n, n, 12, [], [], dt)
+    (A, At), keep = _views(S, dt)
+    t = torch.float32 if dt == np.float32 else torch.float64
+    V, W, Tb = (torch.zeros((2, n), dtype=t, device="cuda") for _ in range(3))
+    Tb[0] = 1.0
+    xrm, z = (torch.zeros((n, 8), dtype=t, device="cuda") for _ in range(2))
+    Ht, Sm, sprev = (torch.zeros((LD, LD), dtype=torch.float64, device="cuda") for _ in range(3))
+    flags = torch.zeros(48, dtype=torch.int32, device="cuda")
+    for skew in (1.0, 4.0, 8.0, 16.0):
+        A.skew = At.skew = skew
+        ok = _call(lib, EXPAND % ("f" if dt == np.float32 else "d"),
+                   [A, At, 1, 0, 0, 0, Tb, V, W, Tb, xrm, z, Ht, Sm, sprev, LD, flags,
+                    C.c_void_p(flags.data_ptr() + 160)], C.c_bool)
+        line = n * 8 * (2 / 2e6 if dt == np.float64 else 1e-6) + 2 * skew * S.nnz * 3 * np.dtype(dt).itemsize / 30e6
+        assert ok == (line <= 1.0) and (ok or skew > 1.0), line
